@@ -110,7 +110,9 @@ typedef struct {
   int64_t mem_budget;    /* device bytes the handle may allocate; 0 = no limit */
   int32_t tile_kz;       /* z planes per thread block of the full step kernel (FP32 tiles
                             holding FEM-cube or free nodes; every FP64 tile); tuning:
-                            0 = library default (16 for n >= 128, else 8), else 2..n */
+                            0 = library default (FP32: 16 for n >= 128, else 8; FP64: 1..16
+                            planes, as many as leave an item for every resident thread
+                            block of the GPU), else 2..n */
   int32_t forward_only;  /* nonzero: keep neither the E history nor snapshots (for
                             data generation); ddfd_adjoint then fails with DDFD_E_STATE */
   /* fem_kind = DDFD_FEM_MESH: the tetrahedra of the FEM cube [a, b]^3, a locally

@@ -67,6 +67,18 @@ void dfree(ddfd_problem *p, void *ptr) {
     }
 }
 
+// FP64: the step is bound by the SMs' FP64 units, so a small grid is cut into
+// about as many items as the chip holds CTAs (152 SMs x 2), down to one plane
+// each; beyond that deeper items save halo planes and the Gauss-law term's
+// extra layer per item.
+int default_kz(int n, int fp32, int count) {
+  if (fp32) return n >= 128 ? 16 : 8;
+  const long long cols = (long long)step_tiles_x(n, false) * step_tiles_y(n, false) * count;
+  const long long kz = (cols * n + 303) / 304;
+  return (int)std::min<long long>(std::max<long long>(kz, 1), 16);
+}
+int default_kz_lean(int n) { return n >= 128 ? 16 : 8; }
+
 std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &ps, int kz, int kz_lean,
                                       int *n_full) {
   const int n = ps[0]->n;
@@ -908,8 +920,8 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   p->fp32 = cfg->precision == DDFD_FP32;
   p->esz = p->fp32 ? 4 : 8;
   p->stream = (cudaStream_t)cfg->stream;
-  p->kz = cfg->tile_kz ? cfg->tile_kz : (p->n >= 128 ? 16 : 8);
-  p->kz_lean = cfg->tile_kz_lean ? cfg->tile_kz_lean : (p->n >= 128 ? 16 : 8);
+  p->kz = ext ? ext->kz : cfg->tile_kz ? cfg->tile_kz : default_kz(p->n, p->fp32, 1);
+  p->kz_lean = ext ? ext->kz_lean : cfg->tile_kz_lean ? cfg->tile_kz_lean : default_kz_lean(p->n);
 
   auto bail = [&](int code) {
     g_create_err = p->err;

@@ -387,8 +387,8 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   b->esz = b->fp32 ? 4 : 8;
   b->seg = seg;
   b->stream = (cudaStream_t)cfgs[0].stream;
-  b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : (b->n >= 128 ? 16 : 8);
-  b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : (b->n >= 128 ? 16 : 8);
+  b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : default_kz(b->n, b->fp32, std::min(count, BATCH_MAX));
+  b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : default_kz_lean(b->n);
   auto bail = [&](int code, const std::string &m) {
     ddfd::set_thread_error(m);
     destroy_batch(b);
@@ -425,8 +425,6 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   for (int i = 0; i < count; ++i) {
     ddfd_config c = cfgs[i];
     c.stream = cfgs[0].stream;
-    c.tile_kz = b->kz;
-    c.tile_kz_lean = b->kz_lean;
     MemberSlot ms;
     for (int q = 0; q < 2; ++q) {
       ms.E[q] = (char *)b->E[q] + i * fb;
@@ -435,6 +433,8 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
     ms.kcoef = (char *)b->kcoef + i * fb;
     ms.batch = b;
     ms.slot = i;
+    ms.kz = b->kz;
+    ms.kz_lean = b->kz_lean;
     ddfd_problem *p = nullptr;
     const int st = create_impl(&c, &ms, &p);
     if (st) return bail(st, "member " + std::to_string(i) + ": " + thread_error());

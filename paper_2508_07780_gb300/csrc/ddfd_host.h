@@ -182,6 +182,7 @@ struct MemberSlot {
   void *E[2], *Mu[2], *kcoef;
   ddfd_batch *batch;
   int slot;
+  int kz, kz_lean;  // the batch's tile depths
 };
 
 // Message of the last failing handle-less call in this thread.
@@ -209,6 +210,11 @@ int bfail(ddfd_batch *b, int code, const std::string &m);
 // dfree releases one such allocation early.
 int dalloc(ddfd_problem *p, size_t bytes, void **out);
 void dfree(ddfd_problem *p, void *ptr);
+
+// Default z depths of the step kernels' items (tile_kz = 0, tile_kz_lean = 0)
+// for `count` problems of n^3 nodes.
+int default_kz(int n, int fp32, int count);
+int default_kz_lean(int n);
 
 // Dispatch order of one step launch over the problems `ps` (stacked in that
 // order), in z slabs (one problem's z range over a set of its tile columns,

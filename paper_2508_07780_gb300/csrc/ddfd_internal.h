@@ -162,6 +162,11 @@ constexpr int ITEM_MAX_NZ = 64;
 // before any launch or capture).
 cudaError_t prepare_step_kernels();
 
+// FP64 (ddfd_step64.cu): its part of prepare_step_kernels, and one step.
+cudaError_t prepare_step64_kernels();
+template <bool ADJ, int NB>
+int launch_step64(const StepLaunch<double, NB> &L, cudaStream_t s);
+
 // One step: returns the number of kernels launched (1, or 2 when the FP32
 // tiles are split; the lean launch goes to fk->side when fk has one, else to s).
 template <typename T, int NB>

@@ -11,8 +11,7 @@
 //     (2 CTAs per SM) and the lean kernel, without the block stencil, the
 //     gradient or the coefficient stages, for the finite-difference items
 //     (3 CTAs per SM).
-//   - FP64 (k_step): 32 x 8 tiles, one node per thread, 8 compute warps and
-//     a producer warp, every tile on one kernel.
+//   - FP64: ddfd_step64.cu, 32 x 8 tiles, every tile on one kernel.
 // The planes of the current field (with a one-node halo in y and a
 // 16-byte-aligned halo in x), the centre tile of the previous level, and (on
 // tiles that touch the FEM cube) the coefficient planes are staged into
@@ -47,8 +46,7 @@
 
 #include <cmath>
 
-#include "ddfd_internal.h"
-#include "ddfd_tma.h"
+#include "ddfd_step_common.h"
 
 namespace ddfd {
 
@@ -81,15 +79,6 @@ cudaError_t check_kuhn_blocks(const KuhnBlocks &kb, cudaStream_t) {
   return cudaSuccess;
 }
 
-__device__ __forceinline__ double pulse_value(int kind, double f, double t0, double w, double t) {
-  if (kind == DDFD_SRC_GAUSS) {
-    const double s = t - t0;
-    const double q = s / w;
-    return sin(2.0 * 3.141592653589793 * f * s) * exp(-q * q);
-  }
-  return (t > 0.0 && t < 1.0 / f) ? sin(2.0 * 3.141592653589793 * f * t) : 0.0;
-}
-
 // sum_o B_o v_{i+o} for one node (B = kb / 6), with B_{-o} = B_o; v given as
 // the centre value and the 7 (+o, -o) neighbour pairs already summed.
 template <typename T>
@@ -113,41 +102,6 @@ __device__ __forceinline__ void block_apply(const T v0[3], const T vp[7][3], T o
     out[c] = acc * T(1.0 / 6.0);
   }
 }
-
-__device__ __forceinline__ int face_count(int i, int j, int k, int n, uint32_t abs) {
-  int f = 0;
-  if (i == 0 && (abs & DDFD_ABS_X0)) ++f;
-  if (i == n - 1 && (abs & DDFD_ABS_X1)) ++f;
-  if (j == 0 && (abs & DDFD_ABS_Y0)) ++f;
-  if (j == n - 1 && (abs & DDFD_ABS_Y1)) ++f;
-  if (k == 0 && (abs & DDFD_ABS_BOTTOM)) ++f;
-  if (k == n - 1 && (abs & DDFD_ABS_TOP)) ++f;
-  return f;
-}
-
-template <typename T>
-struct Stage {
-  static constexpr int TX = STEP_TX;
-  static constexpr int TY = StepTile<T>::TY;       // tile rows
-  static constexpr int RPT = TY / 8;               // rows per thread (256 threads = 32 x 8)
-  static constexpr int HX = 16 / (int)sizeof(T);   // x halo: one 16-byte unit
-  static constexpr int BXW = STEP_TX + 2 * HX;     // staged row length
-  static constexpr int ROWS = TY + 2;
-  static constexpr int TXY = STEP_TX * TY;
-  static constexpr int up128(int b) { return (b + 127) / 128 * 128; }
-  static constexpr int E_BYTES = 3 * ROWS * BXW * (int)sizeof(T);  // current level, halo
-  static constexpr int O_BYTES = 3 * TXY * (int)sizeof(T);         // previous level, centre
-  static constexpr int S_BYTES = ROWS * BXW * (int)sizeof(T);      // s = eps - 1, halo
-  static constexpr int Q_BYTES = 2 * TXY * (int)sizeof(T);         // (q1, q2), centre
-  static constexpr int E_OFF = 0;
-  static constexpr int O_OFF = up128(E_BYTES);
-  static constexpr int S_OFF = O_OFF + up128(O_BYTES);
-  static constexpr int Q_OFF = S_OFF + up128(S_BYTES);
-  static constexpr int BYTES = Q_OFF + up128(Q_BYTES);
-  // FP32: 6 stages (3 CTAs per SM); FP64: 4 stages (2 CTAs per SM)
-  static constexpr int RING = sizeof(T) == 4 ? 6 : 4;
-  static constexpr int SMEM = RING * BYTES + 2 * RING * 8 + 128;
-};
 
 // FP32 stage: 32 x 16 tile, each computing thread owns two x-adjacent nodes
 // (so every staged row is read as float2 pairs); 5 stages.  Full kernel
@@ -178,400 +132,6 @@ struct PairStageT {
   static constexpr int SMEM = RING * BYTES + 2 * RING * 8 + RING * 4 + 8 + 128;
 };
 using PairStage = PairStageT<false>;
-
-// Warp roles: warps 0..7 compute, warp 8 stages planes.
-constexpr int STEP_CONSUMERS = 256;
-constexpr int STEP_THREADS = STEP_CONSUMERS + 32;
-
-// Stages plane p = kk - (k0 - 1) of the chunk into slot p % RING and arms the
-// slot's "full" barrier with the byte count: the current level (halo box;
-// mirrored ghost planes at kk = -1 and kk = n), the previous level (centre
-// box, computed planes only) and, on tiles touching the FEM cube, s (halo
-// box, planes a..b) and (q1, q2) (centre box, computed planes a..b).
-template <class S>
-__device__ __forceinline__ void stage_plane(int p, const CUtensorMap *mcur, const CUtensorMap *mold,
-                                            const CUtensorMap *ms, const CUtensorMap *mq, unsigned char *smem,
-                                            uint64_t *bar, int x0, int y0, int k0, int k1, int n, bool tile_fem,
-                                            int a, int b, int ch) {
-  const int slot = p % S::RING;
-  const int kk = k0 - 1 + p;
-  const int ksrc = kk < 0 ? 1 : (kk >= n ? n - 2 : kk);  // mirror ghost planes
-  unsigned char *st = smem + slot * S::BYTES;
-  const bool interior = kk >= k0 && kk < k1;
-  const bool coef = tile_fem && kk >= a && kk <= b;
-  const bool qc = coef && interior;
-  const uint32_t bytes = S::E_BYTES + (interior ? S::O_BYTES : 0) + (coef ? S::S_BYTES : 0) +
-                         (qc ? S::Q_BYTES : 0);
-  uint64_t *bb = &bar[slot];
-  mbar_expect_tx(bb, bytes);
-  tma_load_4d(st + S::E_OFF, mcur, x0 - S::HX, y0 - 1, ksrc, ch, bb);
-  if (interior) tma_load_4d(st + S::O_OFF, mold, x0, y0, kk, ch, bb);
-  if (coef) tma_load_4d(st + S::S_OFF, ms, x0 - S::HX, y0 - 1, kk, ch, bb);
-  if (qc) tma_load_4d(st + S::Q_OFF, mq, x0, y0, kk, ch + 1, bb);
-}
-
-// Producer (one thread): stages plane p = kk - (k0 - 1) of the chunk into
-// slot p % RING once the consumers have released the slot's previous plane
-// (p - RING): the current level (halo box; mirrored ghost planes at kk = -1
-// and kk = n), the previous level (centre box, computed planes only) and, on
-// tiles touching the FEM cube, s (halo box, planes a..b) and (q1, q2)
-// (centre box, computed planes a..b).  Every wait is bounded; on give-up it
-// sets error bit 4 and still waits (bounded) for its issued copies.
-template <class S>
-__device__ __forceinline__ void produce_planes(const CUtensorMap *mcur, const CUtensorMap *mold,
-                                               const CUtensorMap *ms, const CUtensorMap *mq,
-                                               unsigned char *smem, uint64_t *bar, uint64_t *emp, int x0,
-                                               int y0, int k0, int k1, int n, bool tile_fem, int a, int b,
-                                               int ch, uint32_t spin, int *err) {
-  const int nplanes = k1 - k0 + 2;
-  int p = 0;
-  bool ok = true;
-  for (; p < nplanes; ++p) {
-    const int slot = p % S::RING;
-    // plane p reuses the slot of plane p - RING, whose release is completion
-    // number p/RING - 1 of that slot's empty barrier
-    if (p >= S::RING && !mbar_wait_bounded(&emp[slot], (uint32_t)((p / S::RING - 1) & 1), spin)) {
-      ok = false;
-      break;
-    }
-    stage_plane<S>(p, mcur, mold, ms, mq, smem, bar, x0, y0, k0, k1, n, tile_fem, a, b, ch);
-  }
-  if (!ok) atomicOr(err, 4);
-  // every issued plane must land before the CTA can retire (bounded)
-  const int first = p > S::RING ? p - S::RING : 0;
-  for (int q = first; q < p; ++q)
-    mbar_wait_bounded(&bar[q % S::RING], (uint32_t)((q / S::RING) & 1), spin);
-}
-
-// Tiles per axis of the launch grid (device side of step_tiles_x / _y).  x
-// tiles of the FP32 step kernel: with n = 32 m + 1 the last column is updated
-// by the last of m tiles (k_step_pair's x tail) instead of by a tile of its own.
-__host__ __device__ constexpr int tiles_pair_x(int n) { return n % STEP_TX == 1 ? n / STEP_TX : (n + STEP_TX - 1) / STEP_TX; }
-template <typename T>
-__device__ __forceinline__ int step_tiles_dev_x(int n) {
-  return sizeof(T) == 4 ? tiles_pair_x(n) : (n + STEP_TX - 1) / STEP_TX;
-}
-template <typename T>
-__device__ __forceinline__ int step_tiles_dev_y(int n) {
-  return (n + StepTile<T>::TY - 1) / StepTile<T>::TY;
-}
-
-// Tile of this CTA: (problem of the launch, tile x, tile y) and its planes
-// [k0, k1), from the launch's dispatch order if it has one, else from the 3-D
-// grid (z chunks of kz planes).
-struct CtaTile {
-  int prob, tx, ty, k0, k1;
-};
-template <typename LT>
-__device__ __forceinline__ CtaTile cta_tile(const LT &L) {
-  CtaTile t;
-  if (L.items) {
-    const uint32_t it = L.items[blockIdx.x];
-    t.tx = (int)(it & 31u);
-    t.ty = (int)((it >> 5) & 127u);
-    t.k0 = (int)((it >> 12) & 1023u);
-    t.k1 = t.k0 + (int)((it >> 22) & 63u) + 1;
-    t.prob = (int)(it >> 28);
-  } else {
-    t.tx = (int)blockIdx.x;
-    t.ty = (int)blockIdx.y;
-    t.prob = (int)blockIdx.z / L.zchunks;
-    const int zc = (int)blockIdx.z - t.prob * L.zchunks;
-    const int kz = L.p[sizeof(L.p) == sizeof(L.p[0]) ? 0 : t.prob].kz;
-    t.k0 = zc * kz;
-    t.k1 = t.k0 + kz;
-  }
-  return t;
-}
-
-// Forward detector sampling of E^n (read-only in the step kernels): the CTAs
-// that own the bottom planes (k0 = 0) of a tile column, one per column
-// whatever the z chunking, share the 3 n_det values by the first 256 threads'
-// index within the column grid.
-template <typename T>
-__device__ __forceinline__ void sample_detectors(const StepParams<T> &P, const CtaTile &ct, int tid) {
-  if (P.n_det <= 0 || ct.k0 != 0 || tid >= STEP_CONSUMERS) return;
-  const int n = P.n;
-  const int gx = step_tiles_dev_x<T>(n), gy = step_tiles_dev_y<T>(n);
-  const long long nb = (long long)gx * gy * STEP_CONSUMERS;
-  for (long long t = ((long long)ct.tx + (long long)gx * ct.ty) * STEP_CONSUMERS + tid; t < 3LL * P.n_det; t += nb) {
-    const int d = (int)(t / 3), c = (int)(t - 3LL * d);
-    P.trace_n[t] = (double)P.cur[c * P.cs + P.det_node[d]];
-  }
-}
-
-template <typename T, bool ADJ, int NB>
-__global__ void __launch_bounds__(STEP_THREADS, sizeof(T) == 4 ? 3 : 2)
-    k_step(const __grid_constant__ StepLaunch<T, NB> L) {
-  using S = Stage<T>;
-  // problem of this CTA (uniform), its tile and z chunk
-  const CtaTile ct = cta_tile(L);
-  const StepParams<T> &P = L.p[NB == 1 ? 0 : ct.prob];
-  constexpr int RE = S::ROWS * S::BXW;  // component stride of a staged plane
-  constexpr int BW = S::BXW;
-  // 128-byte aligned stage base, computed in the shared window so that the
-  // compiler keeps every stage access a shared-memory access
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-  uint64_t *bar = (uint64_t *)(smem + S::RING * S::BYTES);  // "full": plane landed
-  uint64_t *emp = bar + S::RING;                             // "empty": consumers released it
-  const int n = P.n;
-  const int tid = threadIdx.x;
-
-  if (!ADJ) sample_detectors(P, ct, tid);
-
-  const int tx = tid & 31, ty = tid >> 5;
-  // one CTA per (tile, z range): planes k0-1 .. k1 are staged, plane index
-  // p = kk - (k0 - 1) in slot p % RING
-  const int x0 = ct.tx * STEP_TX, y0 = ct.ty * S::TY;
-  const int k0 = ct.k0;
-  if (k0 >= n) return;  // uniform per CTA
-  const int k1 = min(ct.k1, n);
-  const bool tile_fem = x0 <= P.b - 1 && x0 + STEP_TX - 1 >= P.a + 1 && y0 <= P.b - 1 &&
-                        y0 + S::TY - 1 >= P.a + 1;
-
-  if (tid == 0) {
-    for (int s = 0; s < S::RING; ++s) {
-      mbar_init(&bar[s], 1);
-      mbar_init(&emp[s], STEP_CONSUMERS / 32);
-    }
-    mbar_fence_init();
-    tma_prefetch_desc(&L.cur);
-    tma_prefetch_desc(&L.old);
-    tma_prefetch_desc(&L.s);
-    tma_prefetch_desc(&L.q);
-  }
-  __syncthreads();
-
-  if (tid >= STEP_CONSUMERS) {
-    if (tid == STEP_CONSUMERS)
-      produce_planes<S>(&L.cur, &L.old, &L.s, &L.q, smem, bar, emp, x0, y0, k0, k1, n, tile_fem, P.a, P.b,
-                        P.chan, P.spin_limit, P.err);
-    return;
-  }
-
-  const long long plane = (long long)P.px * n;
-  const uint32_t cs = (uint32_t)P.cs;
-  const uint32_t sides = (P.abs_now | P.abs_next) & (DDFD_ABS_X0 | DDFD_ABS_X1 | DDFD_ABS_Y0 | DDFD_ABS_Y1);
-  int wq = 0, wslot = 0;   // planes waited so far, slot of the next wait
-  uint32_t wphase = 0;     // parity of the next wait
-  int sm1 = 0, s0 = 1, sp1 = 2;  // slots of planes p-1, p, p+1 (p = k - k0 + 1)
-  {
-    // per-row constants
-    const int x = x0 + tx;
-    int y[S::RPT], ci[S::RPT], oi[S::RPT], dym[S::RPT], dyp[S::RPT];
-    bool live[S::RPT], colfem[S::RPT], colfree[S::RPT], colbnd[S::RPT];
-    T *out[S::RPT];
-#pragma unroll
-    for (int r = 0; r < S::RPT; ++r) {
-      const int yy = ty + 8 * r;
-      y[r] = y0 + yy;
-      ci[r] = (yy + 1) * BW + (tx + S::HX);
-      oi[r] = yy * STEP_TX + tx;
-      dym[r] = (y[r] == 0) ? BW : -BW;
-      dyp[r] = (y[r] == n - 1) ? -BW : BW;
-      live[r] = x < n && y[r] < n;
-      colfem[r] = x > P.a && x < P.b && y[r] > P.a && y[r] < P.b;
-      colfree[r] = x >= P.f0 && x < P.f0 + P.nf && y[r] >= P.f0 && y[r] < P.f0 + P.nf;
-      // side columns need the boundary path only where a side face absorbs
-      colbnd[r] = (x == 0 && (sides & DDFD_ABS_X0)) || (x == n - 1 && (sides & DDFD_ABS_X1)) ||
-                  (y[r] == 0 && (sides & DDFD_ABS_Y0)) || (y[r] == n - 1 && (sides & DDFD_ABS_Y1));
-      out[r] = P.old + (long long)k0 * plane + (long long)P.px * y[r] + x;
-    }
-    const int dxm = (x == 0) ? 1 : -1, dxp = (x == n - 1) ? -1 : 1;
-    T below[S::RPT][3], cen[S::RPT][3];
-
-    for (int k = k0; k < k1; ++k) {
-      const int p = k - k0 + 1;
-      bool ok = true;
-      while (wq <= p + 1) {
-        if (!mbar_wait_bounded(&bar[wslot], wphase, P.spin_limit)) {
-          ok = false;
-          break;
-        }
-        ++wq;
-        if (++wslot == S::RING) {
-          wslot = 0;
-          wphase ^= 1u;
-        }
-      }
-      if (!__all_sync(0xffffffffu, ok)) {  // warp-uniform, so __syncwarp below stays safe
-        if ((tid & 31) == 0) atomicOr(P.err, 4);
-        break;  // the producer times out on the slots we no longer release
-      }
-      const unsigned char *bm1 = smem + sm1 * S::BYTES;
-      const unsigned char *b0 = smem + s0 * S::BYTES;
-      const unsigned char *bp1 = smem + sp1 * S::BYTES;
-      const T *Em = (const T *)(bm1 + S::E_OFF);
-      const T *E0 = (const T *)(b0 + S::E_OFF);
-      const T *Ep = (const T *)(bp1 + S::E_OFF);
-      const T *O0 = (const T *)(b0 + S::O_OFF);
-      const bool kfem = k > P.a && k < P.b;
-      const bool kfree = k >= P.f0 && k < P.f0 + P.nf;
-      // bottom plane: absorbing or plain Neumann; top plane: source, absorbing
-      // face or detector residuals
-      const bool kbnd = (k == 0 && ((P.abs_now | P.abs_next) & DDFD_ABS_BOTTOM)) || k == n - 1;
-#pragma unroll
-      for (int r = 0; r < S::RPT; ++r) {
-        T above[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          if (k == k0) {
-            below[r][c] = Em[c * RE + ci[r]];
-            cen[r][c] = E0[c * RE + ci[r]];
-          }
-          above[c] = Ep[c * RE + ci[r]];
-        }
-        if (live[r]) {
-          const bool fre = colfree[r] && kfree;
-          long long fi = 0;
-          if (fre) fi = (x - P.f0) + (long long)P.nf * ((y[r] - P.f0) + (long long)P.nf * (k - P.f0));
-          T od[3], R[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const T *e = E0 + c * RE + ci[r];
-            od[c] = O0[c * S::TXY + oi[r]];
-            R[c] = T(6) * cen[r][c] - (e[dxp] + e[dxm] + e[dyp[r]] + e[dym[r]] + above[c] + below[r][c]);
-          }
-          // update coefficients: nw = cen + A (cen - od) + Bc cen - Cq tau^2 R
-          T A = T(1), Bc = T(0), Cq = T(1);
-          T sx[3] = {T(0), T(0), T(0)};
-          if (colfem[r] && kfem && P.ebe_r) {
-            // element-by-element rows computed by k_ebe for this step
-            const T *Q0 = (const T *)(b0 + S::Q_OFF);
-            A = Q0[oi[r]];
-            Cq = Q0[S::TXY + oi[r]];
-            const int fm = P.b - P.a - 1;
-            const long long row = (x - P.a - 1) + (long long)fm * ((y[r] - P.a - 1) + (long long)fm * (k - P.a - 1));
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              R[c] = P.ebe_r[c * P.ebe_rows + row];
-              if (ADJ) sx[c] = P.ebe_q[c * P.ebe_rows + row];
-            }
-          } else if (colfem[r] && kfem) {
-            const T *S0 = (const T *)(b0 + S::S_OFF);
-            const T *Q0 = (const T *)(b0 + S::Q_OFF);
-            const int q = ci[r];
-            const T s0v = S0[q];
-            A = Q0[oi[r]];
-            Cq = Q0[S::TXY + oi[r]];
-            T v0[3], vp[7][3], st[3];
-            if (!ADJ) {
-              const T *Sm = (const T *)(bm1 + S::S_OFF);
-              const T *Sp = (const T *)(bp1 + S::S_OFF);
-#pragma unroll
-              for (int c = 0; c < 3; ++c) {
-                const T *e0 = E0 + c * RE, *ep = Ep + c * RE, *em = Em + c * RE;
-                v0[c] = s0v * cen[r][c];
-                vp[0][c] = S0[q + 1] * e0[q + 1] + S0[q - 1] * e0[q - 1];
-                vp[1][c] = S0[q + BW] * e0[q + BW] + S0[q - BW] * e0[q - BW];
-                vp[2][c] = Sp[q] * above[c] + Sm[q] * below[r][c];
-                vp[3][c] = S0[q + 1 + BW] * e0[q + 1 + BW] + S0[q - 1 - BW] * e0[q - 1 - BW];
-                vp[4][c] = Sp[q + 1] * ep[q + 1] + Sm[q - 1] * em[q - 1];
-                vp[5][c] = Sp[q + BW] * ep[q + BW] + Sm[q - BW] * em[q - BW];
-                vp[6][c] = Sp[q + 1 + BW] * ep[q + 1 + BW] + Sm[q - 1 - BW] * em[q - 1 - BW];
-              }
-              block_apply<T>(v0, vp, st);
-#pragma unroll
-              for (int c = 0; c < 3; ++c) R[c] += st[c];
-            } else if (s0v != T(0) || fre) {
-#pragma unroll
-              for (int c = 0; c < 3; ++c) {
-                const T *e0 = E0 + c * RE, *ep = Ep + c * RE, *em = Em + c * RE;
-                v0[c] = cen[r][c];
-                vp[0][c] = e0[q + 1] + e0[q - 1];
-                vp[1][c] = e0[q + BW] + e0[q - BW];
-                vp[2][c] = above[c] + below[r][c];
-                vp[3][c] = e0[q + 1 + BW] + e0[q - 1 - BW];
-                vp[4][c] = ep[q + 1] + em[q - 1];
-                vp[5][c] = ep[q + BW] + em[q - BW];
-                vp[6][c] = ep[q + 1 + BW] + em[q - 1 - BW];
-              }
-              block_apply<T>(v0, vp, sx);
-#pragma unroll
-              for (int c = 0; c < 3; ++c) R[c] += s0v * sx[c];
-            }
-          }
-#pragma unroll
-          for (int c = 0; c < 3; ++c) R[c] *= P.r2;
-          if (colbnd[r] || kbnd) {
-            // boundary node: damping of the absorbing faces, top-face source or
-            // detector residuals
-            const int fn = face_count(x, y[r], k, n, P.abs_now);
-            const T cc = P.cb * T(fn);
-            const T ccn = ADJ ? P.cb * T(face_count(x, y[r], k, n, P.abs_next)) : cc;
-            const T inv = P.inv_tab[fn];  // 1 / (1 + cc)
-            A = (T(1) - ccn) * inv;
-            Bc = (ccn - cc) * inv;
-            Cq = inv;
-            if (!ADJ && k == n - 1 && P.src_on) {
-              if (!P.oblique) {
-                R[1] -= P.src_y;
-              } else {
-                const double v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width,
-                                                           P.t_n - P.delay[x + n * y[r]]);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) R[c] -= (T)(P.pol[c] * v);
-              }
-            }
-            if (ADJ && k == n - 1 && P.n_det > 0) {
-              const int q0 = P.det_ptr[x + n * y[r]], q1 = P.det_ptr[x + n * y[r] + 1];
-              if (q1 > q0) {
-                const double wx = (x == 0 || x == n - 1) ? 0.5 : 1.0;
-                const double wy = (y[r] == 0 || y[r] == n - 1) ? 0.5 : 1.0;
-                const double sc = P.tau2 * P.inv_h3 / (wx * wy * 0.5);
-                double acc[3] = {0.0, 0.0, 0.0};
-                for (int qq = q0; qq < q1; ++qq) {
-                  const int d = P.det_list[qq];
-                  acc[0] += P.res_k[3 * d + 0];
-                  acc[1] += P.res_k[3 * d + 1];
-                  acc[2] += P.res_k[3 * d + 2];
-                }
-#pragma unroll
-                for (int c = 0; c < 3; ++c) R[c] += (T)(sc * acc[c]);
-              }
-            }
-          }
-          T nw[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            nw[c] = cen[r][c] + (A * (cen[r][c] - od[c]) + (Bc * cen[r][c] - Cq * R[c]));
-            out[r][c * cs] = nw[c];
-          }
-          if (fre) {
-            if (!ADJ) {
-            if (P.hist_w)
-#pragma unroll
-              for (int c = 0; c < 3; ++c) P.hist_w[c * P.n_free + fi] = nw[c];
-            } else {
-              T ge = T(0), gs = T(0);
-#pragma unroll
-              for (int c = 0; c < 3; ++c) {
-                const T hv = __ldg(P.hist_r + c * P.n_free + fi);
-                ge += hv * ((nw[c] - T(2) * cen[r][c] + od[c]) + P.r2 * sx[c]);
-                gs += hv * (nw[c] - od[c]);
-              }
-              P.gacc_e[fi] += (double)ge;
-              P.gacc_s[fi] += (double)gs;
-            }
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          below[r][c] = cen[r][c];
-          cen[r][c] = above[c];
-        }
-        out[r] += plane;
-      }
-      // release plane p-1 (its slot) to the producer: one arrival per warp
-      __syncwarp();
-      if ((tid & 31) == 0) mbar_arrive(&emp[sm1]);
-      sm1 = s0;
-      s0 = sp1;
-      sp1 = (sp1 + 1 == S::RING) ? 0 : sp1 + 1;
-    }
-  }
-}
 
 // ---------------------------------------------------------------------------
 // FP32 step kernel, two x-adjacent nodes per thread
@@ -1095,11 +655,6 @@ __global__ void __launch_bounds__(PairMode<ADJ, LEAN>::THREADS, PairMode<ADJ, LE
 }
 
 template <bool ADJ, int NB>
-static cudaError_t set_smem_f64() {
-  return cudaFuncSetAttribute(k_step<double, ADJ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              Stage<double>::SMEM);
-}
-template <bool ADJ, int NB>
 static cudaError_t set_smem_f32() {
   cudaError_t e = cudaFuncSetAttribute(k_step_pair<ADJ, NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        PairStageT<false>::SMEM);
@@ -1111,11 +666,9 @@ static cudaError_t set_smem_f32() {
 cudaError_t prepare_step_kernels() {
   cudaError_t e;
   if ((e = set_smem_f32<false, 1>()) != cudaSuccess || (e = set_smem_f32<true, 1>()) != cudaSuccess ||
-      (e = set_smem_f64<false, 1>()) != cudaSuccess || (e = set_smem_f64<true, 1>()) != cudaSuccess ||
-      (e = set_smem_f32<false, BATCH_MAX>()) != cudaSuccess || (e = set_smem_f32<true, BATCH_MAX>()) != cudaSuccess ||
-      (e = set_smem_f64<false, BATCH_MAX>()) != cudaSuccess || (e = set_smem_f64<true, BATCH_MAX>()) != cudaSuccess)
+      (e = set_smem_f32<false, BATCH_MAX>()) != cudaSuccess || (e = set_smem_f32<true, BATCH_MAX>()) != cudaSuccess)
     return e;
-  return cudaSuccess;
+  return prepare_step64_kernels();
 }
 
 int step_tiles_x(int n, bool fp32) { return fp32 ? tiles_pair_x(n) : (n + STEP_TX - 1) / STEP_TX; }
@@ -1134,8 +687,7 @@ static dim3 step_grid(const StepLaunch<T, NB> &L) {
 
 template <bool ADJ, int NB>
 static int launch_step(const StepLaunch<double, NB> &L, cudaStream_t s, const StepFork *) {
-  k_step<double, ADJ, NB><<<step_grid(L), STEP_THREADS, Stage<double>::SMEM, s>>>(L);
-  return 1;
+  return launch_step64<ADJ, NB>(L, s);
 }
 // FP32: the dispatch order's FEM/free tiles on the full kernel, the others on
 // the lean one, side by side when fk provides a side stream.

@@ -1,0 +1,51 @@
+"""The FP64 step kernels (csrc/ddfd_step64.cu) where their tiling can go wrong,
+against the oracle: one to three tiles and a ragged rest per axis, FEM cubes
+that fill the grid or lie across the edges of tiles and of z ranges, every z
+depth from one plane up, and depths of several planes that start or end
+inside the cube.
+
+Bar: relative L2 1e-12 on traces, fields, mu, J and the gradient, the bar of the FP64
+path (a few hundred steps of a scheme whose rounding is 1e-16 a step)."""
+import numpy as np
+import pytest
+
+from helpers import capture_steps, rel_l2, run_gpu, run_oracle
+from synth import workload
+
+pytestmark = pytest.mark.gpu
+
+# n, fem_n (n - 2: the cube's rows start two nodes from the boundary)
+GRIDS = [(7, 5), (9, 7), (10, 7), (15, 13), (16, 14), (17, 15), (19, 8), (28, 26), (29, 17), (33, 31), (34, 13)]
+
+
+@pytest.fixture(scope="module")
+def reference():
+    from paper_2508_07780_gb300 import build
+    build.build()
+    seen = {}
+
+    def get(n, fem):
+        if (n, fem) not in seen:
+            w = workload("tiny", n=n, fem_n=fem, n_steps=3 * n // 2 + 20, seed=n, dir_seed=n, det_per_side=3)
+            e, m = capture_steps(w.n_steps)
+            seen[n, fem] = (w, e, m, run_oracle(w, keep_e=e, keep_mu=m, absorbing=1 | 2 | 8 | 16))
+        return seen[n, fem]
+    return get
+
+
+@pytest.mark.parametrize("n,fem", GRIDS)
+def test_fp64_step_at_tile_edges(reference, n, fem):
+    w, e, m, ref = reference(n, fem)
+    first = None
+    for kz in (0, 2, 3, n - 1):
+        out = run_gpu(w, ref["eobs"], precision="fp64", keep_e=e, keep_mu=m, absorbing_faces=1 | 2 | 8 | 16, tile_kz=kz)
+        assert rel_l2(out["trace"], ref["trace"]) <= 1e-12
+        for k in e:
+            assert rel_l2(out["E"][k], ref["E"][k]) <= 1e-12, (kz, k)
+        for k in m:
+            assert rel_l2(out["mu"][k], ref["mu"][k]) <= 1e-12, (kz, k)
+        assert abs(out["J"] - ref["J"]) <= 1e-12 * abs(ref["J"])
+        assert rel_l2(out["g_eps"], ref["g_eps"]) <= 1e-12 and rel_l2(out["g_sig"], ref["g_sig"]) <= 1e-12
+        if first is not None:  # the depth changes no bit
+            assert np.array_equal(out["trace"], first["trace"]) and np.array_equal(out["g_eps"], first["g_eps"])
+        first = first or out
