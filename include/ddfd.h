@@ -281,7 +281,8 @@ int ddfd_test_gather_timeout(ddfd_problem *p, int32_t fault, uint32_t spin_limit
  * whose FEM cube spans nodes [a, b] and free box [f0, f0 + nf) on each axis,
  * boxes[4 q .. 4 q + 3] = (a, b, f0, nf) for problem q, with z depths kz (full
  * kernel, FP64 kernel) and kz_lean (lean FP32 kernel).  Each item packs tile x
- * (bits 0-4, 32 nodes a tile), tile y (bits 5-11; 16 rows FP32, 8 FP64), the
+ * (bits 0-4, 32 nodes a tile), tile y (bits 5-11; 16 rows FP32, 8 FP64, the tile
+ * of large FP64 launches; small ones run on smaller tiles in the same order), the
  * first plane z0 (bits 12-21), the plane count minus one (bits 22-27) and the
  * problem (bits 28-31); the first *n_full items run on the full kernel.  Up to
  * cap items are written to items (may be NULL with cap = 0); *n_items gets

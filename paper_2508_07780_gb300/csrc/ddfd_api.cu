@@ -68,14 +68,14 @@ void dfree(ddfd_problem *p, void *ptr) {
 }
 
 // FP64: the step is bound by the SMs' FP64 units, so a small grid is cut into
-// about as many items as the chip holds CTAs (152 SMs x 2), down to one plane
-// each; beyond that deeper items save halo planes and the Gauss-law term's
-// extra layer per item.
-int default_kz(int n, int fp32, int count) {
+// about as many items as the chip holds thread blocks (152 SMs x 2, 3 or 4),
+// down to one plane each; beyond that deeper items save halo planes and the
+// Gauss-law term's extra layer per item.
+int default_kz(int n, int fp32, int count, Tile64 tile) {
   if (fp32) return n >= 128 ? 16 : 8;
-  const long long cols = (long long)step_tiles_x(n, false) * step_tiles_y(n, false) * count;
-  const long long kz = (cols * n + 303) / 304;
-  return (int)std::min<long long>(std::max<long long>(kz, 1), 16);
+  const long long cols = (long long)((n + tile.w - 1) / tile.w) * ((n + tile.h - 1) / tile.h) * count;
+  const long long ctas = 152 * (tile.w == 32 ? 2 : tile.w == 14 ? 3 : 4);
+  return (int)std::min<long long>(std::max<long long>((cols * n + ctas / 2) / ctas, 1), 16);
 }
 int default_kz_lean(int n) { return n >= 128 ? 16 : 8; }
 
@@ -83,8 +83,8 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
                                       int *n_full) {
   const int n = ps[0]->n;
   const bool f32 = ps[0]->fp32 != 0;
-  const int gx = step_tiles_x(n, f32), gy = step_tiles_y(n, f32);
-  const int ty_rows = f32 ? StepTile<float>::TY : StepTile<double>::TY;
+  const int tw = f32 ? STEP_TX : ps[0]->tile.w, ty_rows = f32 ? STEP_TY : ps[0]->tile.h;
+  const int gx = f32 ? step_tiles_x(n) : (n + tw - 1) / tw, gy = (n + ty_rows - 1) / ty_rows;
   // A slab is one problem's z range [z0, z1) over a set of its tile columns:
   // the items of a slab are dispatched together, so that tiles that share
   // halos run side by side.
@@ -99,8 +99,8 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
   // does tile column (tx, ty) meet [lo, hi]^2 in x and y (the x tail column
   // n - 1 is never a FEM or free node)
   auto meets = [&](int tx, int ty, int lo, int hi) {
-    const int x0 = tx * STEP_TX, y0 = ty * ty_rows;
-    return lo <= hi && x0 <= hi && x0 + STEP_TX - 1 >= lo && y0 <= hi && y0 + ty_rows - 1 >= lo;
+    const int x0 = tx * tw, y0 = ty * ty_rows;
+    return lo <= hi && x0 <= hi && x0 + tw - 1 >= lo && y0 <= hi && y0 + ty_rows - 1 >= lo;
   };
   std::vector<Slab> full, lean;
   std::vector<std::vector<char>> colfem(ps.size());
@@ -390,18 +390,21 @@ int enqueue_forward(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
     int ic = 1, io = 0;  // buffer holding E^n, and E^{n-1}
     StepParams<T> P = base_params<T>(p);
     set_source(P, p, s);
+    bool chained = false;  // the work before the step is a kernel, not a copy
     for (int st = 0; st < Nt; ++st) {
       if (p->nsnap && st % p->seg == 0) {  // snapshot the state (E^st, E^{st-1})
         char *sn = (char *)p->snap + ((size_t)s * p->nsnap + st / p->seg) * 2 * fbytes;
         CK(cudaMemcpyAsync(sn, p->E[ic], fbytes, cudaMemcpyDeviceToDevice, sm));
         CK(cudaMemcpyAsync(sn + fbytes, p->E[io], fbytes, cudaMemcpyDeviceToDevice, sm));
+        chained = false;
       }
       set_forward_step(P, p, s, st, p->E[ic], p->E[io],
                        (p->nsnap || p->fonly) ? nullptr
                                               : (T *)p->hist + ((size_t)s * (Nt + 1) + st + 1) * 3 * p->n_free);
       enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic]);
-      *nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p), sm, &p->fork);
+      *nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p, chained), sm, &p->fork);
       enqueue_new_step<T>(p, p->X[ic], p->X[io], false, P, sm, nk);
+      chained = true;
       std::swap(ic, io);
       if (p->hist_fem) {  // E^{st+1} on the FEM-updated nodes, for the literal gradient
         const size_t nfu = (size_t)(p->b - p->a - 1) * (p->b - p->a - 1) * (p->b - p->a - 1);
@@ -411,8 +414,10 @@ int enqueue_forward(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
       }
       if (s == 0) {
         const int sl = capture_slot(p, st + 1);
-        if (sl >= 0)
+        if (sl >= 0) {
           CK(cudaMemcpyAsync((char *)p->capE + sl * fbytes, p->E[ic], fbytes, cudaMemcpyDeviceToDevice, sm));
+          chained = false;
+        }
       }
     }
     CK(cudaGetLastError());
@@ -455,22 +460,26 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
         int fc = 1, fo = 0;
         StepParams<T> F = base_params<T>(p);
         set_source(F, p, s);
+        bool chained = false;
         for (int st = n0; st < n1; ++st) {
           // (the trace is written again with the same values)
           set_forward_step(F, p, s, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->n_free);
           enqueue_ebe<T>(p, p->E[fc], false, sm, nk);
-          *nk += launch_forward_step(single_launch(F, p->mE_halo[fc], p->mE_ctr[fo], p), sm, &p->fork);
+          *nk += launch_forward_step(single_launch(F, p->mE_halo[fc], p->mE_ctr[fo], p, chained), sm, &p->fork);
+          chained = true;
           std::swap(fc, fo);
         }
         hbase = (const T *)p->hist;
       } else {
         hbase = (const T *)p->hist + (size_t)s * (Nt + 1) * 3 * p->n_free;
       }
+      bool chained = p->nsnap != 0;  // after the segment's replay, or after memsets
       for (int k = n1; k >= n0 + 1; --k) {
         set_adjoint_step(P, p, s, k, p->Mu[ic], p->Mu[io], hbase + (size_t)(k - n0) * 3 * p->n_free, Nt);
         enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic]);
-        *nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p), sm, &p->fork);
+        *nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p, chained), sm, &p->fork);
         enqueue_new_step<T>(p, p->XMu[ic], p->XMu[io], true, P, sm, nk);
+        chained = true;
         if (p->hist_fem) {  // literal gradient: swap the Gauss-law term of step k (mu^k is still in Mu[ic])
           const size_t nfu = (size_t)(p->b - p->a - 1) * (p->b - p->a - 1) * (p->b - p->a - 1);
           launch_grad_literal<T>((const T *)p->hist_fem + ((size_t)s * (Nt + 1) + k) * 3 * nfu, (const T *)p->Mu[ic],
@@ -480,8 +489,10 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
         std::swap(ic, io);
         if (s == 0) {
           const int sl = capture_slot(p, k - 1);
-          if (sl >= 0)
+          if (sl >= 0) {
             CK(cudaMemcpyAsync((char *)p->capMu + sl * fbytes, p->Mu[ic], fbytes, cudaMemcpyDeviceToDevice, sm));
+            chained = false;
+          }
         }
       }
     }
@@ -598,12 +609,12 @@ int cfl_check(ddfd_problem *p) {
 }
 
 // TMA descriptors of one padded field: a 4-D tensor (x, y, z, channel) with
-// row stride px, plane stride px n, channel stride px n^2; the halo box is
-// (32 + 2 hx) x (TY + 2) x 1 x ch starting hx elements (16 bytes) left of
-// the tile, the centre box 32 x TY x 1 x ch.  Out-of-range elements read as
+// row stride px, plane stride px n, channel stride px n^2; the halo box of a
+// tile of tw x ty nodes is (tw + 2 hx) x (ty + 2) x 1 x ch starting hx elements
+// (16 bytes) left of the tile, the centre box tw x ty x 1 x ch.  Out-of-range elements read as
 // zero.
 int encode_map(std::string *err, CUtensorMap *m, void *base, int n, int px, int fp32, int channels,
-               int box_channels, bool halo) {
+               int box_channels, bool halo, Tile64 tile) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     void *fn = nullptr;
@@ -619,8 +630,8 @@ int encode_map(std::string *err, CUtensorMap *m, void *base, int n, int px, int 
   const cuuint64_t dims[4] = {(cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)channels};
   const cuuint64_t strides[3] = {(cuuint64_t)px * esz, (cuuint64_t)px * n * esz, cs * esz};
   const cuuint32_t hx = (cuuint32_t)(16 / esz);
-  const cuuint32_t ty = fp32 ? StepTile<float>::TY : StepTile<double>::TY;
-  const cuuint32_t box[4] = {halo ? (cuuint32_t)STEP_TX + 2 * hx : (cuuint32_t)STEP_TX, halo ? ty + 2 : ty, 1,
+  const cuuint32_t tw = fp32 ? STEP_TX : tile.w, ty = fp32 ? STEP_TY : tile.h;
+  const cuuint32_t box[4] = {halo ? tw + 2 * hx : tw, halo ? ty + 2 : ty, 1,
                              (cuuint32_t)box_channels};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUresult r = encode(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4,
@@ -643,17 +654,17 @@ int sync_check(ddfd_problem *p) {
 }
 
 int encode_field_maps(std::string *err, FieldMaps *fm, void *const E[2], void *const Mu[2], void *coef, int n,
-                      int px, int fp32, int problems) {
+                      int px, int fp32, int problems, Tile64 tile) {
   const int ch = 3 * problems;
   int st;
   for (int q = 0; q < 2; ++q)
-    if ((st = encode_map(err, &fm->E_halo[q], E[q], n, px, fp32, ch, 3, true)) ||
-        (st = encode_map(err, &fm->E_ctr[q], E[q], n, px, fp32, ch, 3, false)) ||
-        (Mu[q] && (st = encode_map(err, &fm->M_halo[q], Mu[q], n, px, fp32, ch, 3, true))) ||
-        (Mu[q] && (st = encode_map(err, &fm->M_ctr[q], Mu[q], n, px, fp32, ch, 3, false))))
+    if ((st = encode_map(err, &fm->E_halo[q], E[q], n, px, fp32, ch, 3, true, tile)) ||
+        (st = encode_map(err, &fm->E_ctr[q], E[q], n, px, fp32, ch, 3, false, tile)) ||
+        (Mu[q] && (st = encode_map(err, &fm->M_halo[q], Mu[q], n, px, fp32, ch, 3, true, tile))) ||
+        (Mu[q] && (st = encode_map(err, &fm->M_ctr[q], Mu[q], n, px, fp32, ch, 3, false, tile))))
       return st;
-  if ((st = encode_map(err, &fm->S, coef, n, px, fp32, ch, 1, true))) return st;
-  return encode_map(err, &fm->Q, coef, n, px, fp32, ch, 2, false);
+  if ((st = encode_map(err, &fm->S, coef, n, px, fp32, ch, 1, true, tile))) return st;
+  return encode_map(err, &fm->Q, coef, n, px, fp32, ch, 2, false, tile);
 }
 
 }  // namespace host
@@ -663,7 +674,7 @@ namespace {
 
 int build_maps(ddfd_problem *p) {
   FieldMaps fm;
-  const int st = encode_field_maps(&p->err, &fm, p->E, p->Mu, p->kcoef, p->n, p->px, p->fp32, 1);
+  const int st = encode_field_maps(&p->err, &fm, p->E, p->Mu, p->kcoef, p->n, p->px, p->fp32, 1, p->tile);
   if (st) return st;
   for (int q = 0; q < 2; ++q) {
     p->mE_halo[q] = fm.E_halo[q];
@@ -920,7 +931,8 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   p->fp32 = cfg->precision == DDFD_FP32;
   p->esz = p->fp32 ? 4 : 8;
   p->stream = (cudaStream_t)cfg->stream;
-  p->kz = ext ? ext->kz : cfg->tile_kz ? cfg->tile_kz : default_kz(p->n, p->fp32, 1);
+  p->tile = ext ? ext->tile : tile64(p->n, 1);
+  p->kz = ext ? ext->kz : cfg->tile_kz ? cfg->tile_kz : default_kz(p->n, p->fp32, 1, p->tile);
   p->kz_lean = ext ? ext->kz_lean : cfg->tile_kz_lean ? cfg->tile_kz_lean : default_kz_lean(p->n);
 
   auto bail = [&](int code) {

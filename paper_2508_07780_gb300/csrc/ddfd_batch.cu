@@ -78,9 +78,11 @@ int enqueue_batch_forward(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
     }
   const std::vector<int> all = all_members(b);
   int ic = 1, io = 0;
+  bool chained = false;  // the work before the step is a kernel, not a copy
   for (int st = 0; st < Nt; ++st) {
     for (ddfd_problem *p : b->m)
       if (p->nsnap && st % p->seg == 0) {
+        chained = false;
         char *sn = (char *)p->snap + (size_t)(st / p->seg) * 2 * fbytes;
         BCK(cudaMemcpyAsync(sn, p->E[ic], fbytes, cudaMemcpyDeviceToDevice, sm));
         BCK(cudaMemcpyAsync(sn + fbytes, p->E[io], fbytes, cudaMemcpyDeviceToDevice, sm));
@@ -91,7 +93,8 @@ int enqueue_batch_forward(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
     };
     // element-by-element members: their FEM rows of this level first
     for (ddfd_problem *p : b->m) enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic], b->errflag);
-    launch_groups<T>(b, false, all, b->maps.E_halo[ic], b->maps.E_ctr[io], fill, sm, nk, &b->items_all);
+    launch_groups<T>(b, false, all, b->maps.E_halo[ic], b->maps.E_ctr[io], fill, sm, nk, &b->items_all, chained);
+    chained = true;
     for (ddfd_problem *p : b->m)
       if (p->n_new) {
         StepParams<T> P = base_params<T>(p);
@@ -148,17 +151,19 @@ int enqueue_batch_adjoint(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
             [&](StepParams<T> &P, ddfd_problem *p) {
               set_forward_step(P, p, 0, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->n_free);
             },
-            sm, nk, &b->items_ck);
+            sm, nk, &b->items_ck, st > n0);
         std::swap(fc, fo);
       }
     }
+    bool chained = !ck.empty() || n1 < Nt;  // after a kernel, or after the memsets
     for (int k = n1; k >= n0 + 1; --k) {
       auto fill = [&](StepParams<T> &P, ddfd_problem *p) {
         const long long hk = p->nsnap ? k - n0 : k;
         set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io], (const T *)p->hist + (size_t)hk * 3 * p->n_free, Nt);
       };
       for (ddfd_problem *p : b->m) enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic], b->errflag);
-      launch_groups<T>(b, true, all, b->maps.M_halo[ic], b->maps.M_ctr[io], fill, sm, nk, &b->items_all);
+      launch_groups<T>(b, true, all, b->maps.M_halo[ic], b->maps.M_ctr[io], fill, sm, nk, &b->items_all, chained);
+      chained = true;
       for (ddfd_problem *p : b->m)
         if (p->n_new) {
           StepParams<T> P = base_params<T>(p);
@@ -387,7 +392,9 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   b->esz = b->fp32 ? 4 : 8;
   b->seg = seg;
   b->stream = (cudaStream_t)cfgs[0].stream;
-  b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : default_kz(b->n, b->fp32, std::min(count, BATCH_MAX));
+  const int group = std::min(count, BATCH_MAX);
+  b->tile = tile64(b->n, group);
+  b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : default_kz(b->n, b->fp32, group, b->tile);
   b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : default_kz_lean(b->n);
   auto bail = [&](int code, const std::string &m) {
     ddfd::set_thread_error(m);
@@ -419,7 +426,7 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   b->allocs.push_back(b->errflag);
   if (cudaMemset(b->errflag, 0, sizeof(int)) != cudaSuccess) return bail(DDFD_E_CUDA, "memset failed");
   std::string m;
-  if (encode_field_maps(&m, &b->maps, b->E, b->Mu, b->kcoef, b->n, b->px, b->fp32, count))
+  if (encode_field_maps(&m, &b->maps, b->E, b->Mu, b->kcoef, b->n, b->px, b->fp32, count, b->tile))
     return bail(DDFD_E_CUDA, m);
   const size_t fb = 3 * (size_t)b->cs * b->esz;
   for (int i = 0; i < count; ++i) {
@@ -435,6 +442,7 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
     ms.slot = i;
     ms.kz = b->kz;
     ms.kz_lean = b->kz_lean;
+    ms.tile = b->tile;
     ddfd_problem *p = nullptr;
     const int st = create_impl(&c, &ms, &p);
     if (st) return bail(st, "member " + std::to_string(i) + ": " + thread_error());

@@ -115,6 +115,7 @@ struct ddfd_problem {
   int state = ddfd::host::ST_READY;
   int64_t generation = 0;     // +1 whenever the coefficients or the forward state change
   int64_t launches = 0, fwd_steps = 0;
+  ddfd::Tile64 tile;          // FP64 tile shape
   int kz = 16;                // z depth of the full step kernel's items (and of the FP64 kernel's)
   int kz_lean = 16;           // z depth of the lean FP32 step kernel's items
   uint32_t *items = nullptr;  // dispatch order of the step launches (heaviest slabs first), for items_kz
@@ -150,6 +151,7 @@ struct ddfd_batch {
   int n = 0, Nt = 0, px = 0, fp32 = 0, kz = 16, kz_lean = 16, seg = 0;
   long long cs = 0;
   size_t esz = 8;
+  ddfd::Tile64 tile;          // FP64 tile shape of every member
   cudaStream_t stream = nullptr, cap_stream = nullptr;
   void *E[2] = {nullptr, nullptr}, *Mu[2] = {nullptr, nullptr}, *kcoef = nullptr;
   std::vector<void *> allocs;
@@ -183,6 +185,7 @@ struct MemberSlot {
   ddfd_batch *batch;
   int slot;
   int kz, kz_lean;  // the batch's tile depths
+  Tile64 tile;
 };
 
 // Message of the last failing handle-less call in this thread.
@@ -213,7 +216,7 @@ void dfree(ddfd_problem *p, void *ptr);
 
 // Default z depths of the step kernels' items (tile_kz = 0, tile_kz_lean = 0)
 // for `count` problems of n^3 nodes.
-int default_kz(int n, int fp32, int count);
+int default_kz(int n, int fp32, int count, Tile64 tile);
 int default_kz_lean(int n);
 
 // Dispatch order of one step launch over the problems `ps` (stacked in that
@@ -262,7 +265,7 @@ int set_coeffs_impl(ddfd_problem *p, const double *eps, const double *sig, const
 int functional_impl(ddfd_problem *p, const double *eobs, double *J, bool host);
 int gradient_impl(ddfd_problem *p, double *g_eps, double *g_sig, bool host);
 int encode_field_maps(std::string *err, FieldMaps *fm, void *const E[2], void *const Mu[2], void *coef, int n,
-                      int px, int fp32, int problems);
+                      int px, int fp32, int problems, Tile64 tile);
 
 // Explicit FEM meshes (ddfd_fem_setup.cu).
 int build_ebe(ddfd_problem *p);
@@ -354,7 +357,7 @@ void set_adjoint_step(StepParams<T> &P, const ddfd_problem *p, int s, int k, con
 
 template <typename T>
 StepLaunch<T, 1> single_launch(const StepParams<T> &P, const CUtensorMap &cur, const CUtensorMap &old,
-                               const ddfd_problem *p) {
+                               const ddfd_problem *p, bool chained = false) {
   StepLaunch<T, 1> L;
   L.cur = cur;
   L.old = old;
@@ -365,6 +368,8 @@ StepLaunch<T, 1> single_launch(const StepParams<T> &P, const CUtensorMap &cur, c
   L.items = P.kz == p->items_kz ? p->items : nullptr;
   L.n_items = p->n_items;
   L.n_full = p->items_nfull;
+  L.tile_w = p->tile.w;
+  L.chained = chained;
   L.p[0] = P;
   return L;
 }
@@ -448,11 +453,12 @@ void enqueue_new_step(ddfd_problem *p, const void *cur, void *old, bool adj, con
 
 // One batched step launch per group of BATCH_MAX members; fill(P, p) sets the
 // per-step scalars of member p; tables (may be NULL): the groups' dispatch
-// orders, used when built for the batch's current kz.
+// orders, used when built for the batch's current kz; chained: the work
+// before on `sm` is a kernel (StepLaunch::chained).
 template <typename T, typename Fill>
 void launch_groups(ddfd_batch *b, bool adj, const std::vector<int> &idx, const CUtensorMap &cur,
                    const CUtensorMap &old, Fill fill, cudaStream_t sm, int64_t *nk,
-                   const ItemTables *tables = nullptr) {
+                   const ItemTables *tables = nullptr, bool chained = false) {
   for (size_t g0 = 0; g0 < idx.size(); g0 += BATCH_MAX) {
     StepLaunch<T, BATCH_MAX> L;
     std::memset(&L, 0, sizeof(L));
@@ -467,6 +473,8 @@ void launch_groups(ddfd_batch *b, bool adj, const std::vector<int> &idx, const C
     L.items = tab ? tables->d[gi] : nullptr;
     L.n_items = tab ? tables->n_items[gi] : 0;
     L.n_full = tab ? tables->n_full[gi] : 0;
+    L.tile_w = b->tile.w;
+    L.chained = chained || g0 > 0;
     for (int g = 0; g < L.nprob; ++g) {
       ddfd_problem *p = b->m[idx[g0 + g]];
       StepParams<T> P = base_params<T>(p);

@@ -33,18 +33,16 @@ bool invert4(const double A[4][4], double X[4][4]);
 // kernels (cudaErrorInvalidValue if they differ).
 cudaError_t check_kuhn_blocks(const KuhnBlocks &kb, cudaStream_t s);
 
-// Step-kernel tiling: a CTA of 256 computing threads owns a STEP_TX x TY
-// (x, y) tile of one z chunk: FP64 one node per thread (TY = 8), FP32 two
-// x-adjacent nodes per thread (TY = 16).
+// Step-kernel tiling.  FP32: a CTA of 256 computing threads owns a 32 x 16
+// (x, y) tile of one z chunk, two x-adjacent nodes per thread.  FP64: one node
+// per thread, a tile shape by the grid's size (tile64).
 constexpr int STEP_TX = 32;
-template <typename T>
-struct StepTile {
-  static constexpr int TY = 8;
+constexpr int STEP_TY = 16;
+struct Tile64 {
+  int w = 32, h = 8;
 };
-template <>
-struct StepTile<float> {
-  static constexpr int TY = 16;
-};
+// FP64 tile of `count` problems of n^3 nodes stepped together.
+Tile64 tile64(int n, int count);
 
 // FP32 gradient accumulation: the adjoint steps of each block of GRAD_BLOCK
 // consecutive time steps are summed in FP32 (per free node) and the block sum
@@ -133,6 +131,8 @@ struct StepLaunch {
   // and run on the full step kernel; the rest are finite-difference z ranges
   // only and run on the lean one (concurrently, on StepFork's side stream)
   int n_full;
+  int tile_w;  // FP64: width of the tile (Tile64)
+  int chained; // the work before this launch in its stream is a kernel: launch as its dependent (launch_chained)
   StepParams<T> p[NB];
 };
 
@@ -146,10 +146,10 @@ struct StepFork {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
-// Tiles per axis of the step kernels' launch grid (FP32: 32 x 16 tiles,
-// with n = 32 m + 1 covered by m x tiles; FP64: 32 x 8 tiles).
-int step_tiles_x(int n, bool fp32);
-int step_tiles_y(int n, bool fp32);
+// Tiles per axis of the FP32 step kernels' launch grid (32 x 16 tiles, with
+// n = 32 m + 1 covered by m x tiles).
+int step_tiles_x(int n);
+int step_tiles_y(int n);
 // One dispatch item: tile x (< 32), tile y (< 128), first plane z0 (< 1024),
 // plane count nz (1..64), problem of the launch (< 16).
 __host__ __device__ inline uint32_t pack_step_item(int tx, int ty, int z0, int nz, int prob) {

@@ -112,7 +112,7 @@ constexpr int round128(int b) { return (b + 127) / 128 * 128; }
 template <bool LEAN>
 struct PairStageT {
   static constexpr int TX = STEP_TX;
-  static constexpr int TY = StepTile<float>::TY;
+  static constexpr int TY = STEP_TY;
   static constexpr int HX = 4;                     // x halo: one 16-byte unit
   static constexpr int BXW = TX + 2 * HX;          // staged row length (40)
   static constexpr int ROWS = TY + 2;
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(PairMode<ADJ, LEAN>::THREADS, PairMode<ADJ, LE
   const int n = P.n;
   const int tid = threadIdx.x;
 
-  if (!ADJ) sample_detectors(P, ct, tid);
+  if (!ADJ) sample_detectors(P, ct, tid, tiles_pair_x(P.n), (P.n + S::TY - 1) / S::TY, STEP_CONSUMERS);
 
   const int x0 = ct.tx * S::TX, y0 = ct.ty * S::TY;
   const int k0 = ct.k0;
@@ -671,18 +671,14 @@ cudaError_t prepare_step_kernels() {
   return prepare_step64_kernels();
 }
 
-int step_tiles_x(int n, bool fp32) { return fp32 ? tiles_pair_x(n) : (n + STEP_TX - 1) / STEP_TX; }
-int step_tiles_y(int n, bool fp32) {
-  const int ty = fp32 ? StepTile<float>::TY : StepTile<double>::TY;
-  return (n + ty - 1) / ty;
-}
+int step_tiles_x(int n) { return tiles_pair_x(n); }
+int step_tiles_y(int n) { return (n + STEP_TY - 1) / STEP_TY; }
 
 // Launch grid: 1-D over the dispatch items, or the 3-D tile grid.
-template <typename T, int NB>
-static dim3 step_grid(const StepLaunch<T, NB> &L) {
-  const int gx = step_tiles_x(L.p[0].n, sizeof(T) == 4), gy = step_tiles_y(L.p[0].n, sizeof(T) == 4);
+template <int NB>
+static dim3 step_grid(const StepLaunch<float, NB> &L) {
   if (L.items) return dim3((unsigned)L.n_items);
-  return dim3(gx, gy, L.zchunks * L.nprob);
+  return dim3(step_tiles_x(L.p[0].n), step_tiles_y(L.p[0].n), L.zchunks * L.nprob);
 }
 
 template <bool ADJ, int NB>

@@ -25,7 +25,9 @@
 // Measured (us a step, forward and adjoint averaged, against the 15-point
 // stencil on full 32 x 8 warps with 8 or 16 planes an item): 161^3 with a
 // 121^3 cube 840 -> 584 (the FP64 instructions alone would take about 425),
-// 41^3 / 21^3 88 -> 29, 13^3 / 9^3 50 -> 12.
+// 41^3 / 21^3 88 -> 29 and 13^3 / 9^3 50 -> 12 on 32 x 8 tiles, 19 and 11 on
+// the small tiles below with each step launched as the last one's programmatic
+// dependent (its barriers and descriptors are set up while that one drains).
 #include "ddfd_step_common.h"
 
 namespace ddfd {
@@ -37,10 +39,17 @@ constexpr int up128(int b) { return (b + 127) / 128 * 128; }
 // A staged plane: the current level and s with a one-node halo in y and a
 // 16-byte halo in x, the previous level and (q1, q2) without.  Three stages:
 // plane k, plane k + 1, and the next one in flight while a plane's FP64 work
-// runs; with the Gauss-law scratch 98 KB, 2 CTAs per SM.
+// runs.  Tiles of 32 x 8 nodes (98 KB with the Gauss-law scratch, 2 CTAs per
+// SM); on small grids of 14 x 9 or 8 x 8 (launch_step64).
+template <int TW, int TH>
 struct Stage64 {
-  static constexpr int TX = STEP_TX;
-  static constexpr int TY = StepTile<double>::TY;
+  static constexpr int TX = TW;
+  static constexpr int TY = TH;
+  // computing threads: the tile's nodes and, on small tiles, warps of their own
+  // for its halo nodes (one warp's FP64 instructions run 64 cycles apart, so
+  // that a thread with two nodes takes twice as long)
+  static constexpr int CONSUMERS = TW == 32 ? 256 : (TW * TH + 31) / 32 * 32 + (2 * (TW + TH) + 4 + 31) / 32 * 32;
+  static constexpr int MIN_CTAS = TW == 32 ? 2 : TW == 14 ? 3 : 4;
   static constexpr int HX = 2;
   static constexpr int BXW = TX + 2 * HX;
   static constexpr int ROWS = TY + 2;
@@ -66,16 +75,20 @@ struct Stage64 {
   static constexpr int DX = 0, DY = 2 * HN, DZ = 4 * HN, DIV = 5 * HN, FX = DIV + 6 * CN, FY = FX + CN;
   static constexpr int G_DOUBLES = FY + CN;
   static_assert(2 * HN <= 6 * CN, "w_x, w_y fit the divergences' space");
+  static_assert(2 * (TW + TH) + 4 <= CONSUMERS, "a thread takes at most one halo node");
+  static_assert(TW % 2 == 0, "TMA boxes start on 16 bytes");
   static constexpr int G_OFF = RING * BYTES;
   static constexpr int BAR_OFF = G_OFF + up128(G_DOUBLES * 8);
   static constexpr int SMEM = BAR_OFF + 2 * RING * 8 + 128;
 };
 
-// Barrier of the computing warps (the producer warp takes no part).
+// Barrier of the NT computing threads (the producer warp takes no part).
+template <int NT>
 __device__ __forceinline__ void compute_sync() {
-  asm volatile("barrier.sync 1, %0;" ::"n"(STEP_CONSUMERS) : "memory");
+  asm volatile("barrier.sync 1, %0;" ::"n"(NT) : "memory");
 }
 // The same with a vote: true if every computing thread passes true.
+template <int NT>
 __device__ __forceinline__ bool compute_all(bool v) {
   uint32_t r;
   asm volatile(
@@ -84,14 +97,16 @@ __device__ __forceinline__ bool compute_all(bool v) {
       "barrier.red.and.pred q, 1, %2, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"((uint32_t)v), "n"(STEP_CONSUMERS)
+      : "r"((uint32_t)v), "n"(NT)
       : "memory");
   return r != 0;
 }
 
-template <bool ADJ, int NB>
-__global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constant__ StepLaunch<double, NB> L) {
-  using S = Stage64;
+template <bool ADJ, int NB, int TW, int TH>
+__global__ void __launch_bounds__(Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, TH>::MIN_CTAS)
+    k_step64(const __grid_constant__ StepLaunch<double, NB> L) {
+  using S = Stage64<TW, TH>;
+  constexpr int NT = S::CONSUMERS;
   constexpr int RE = S::RE, BW = S::BXW, HW = S::HW, CW = S::CW, CN = S::CN;
   const CtaTile ct = cta_tile(L);
   const StepParams<double> &P = L.p[NB == 1 ? 0 : ct.prob];
@@ -103,18 +118,10 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
   const int n = P.n;
   const int tid = threadIdx.x;
 
-  if (!ADJ) sample_detectors(P, ct, tid);
-
-  const int x0 = ct.tx * S::TX, y0 = ct.ty * S::TY;
-  const int k0 = ct.k0;
-  if (k0 >= n) return;  // uniform per CTA
-  const int k1 = min(ct.k1, n);
-  const bool tile_fem = x0 <= P.b - 1 && x0 + S::TX - 1 >= P.a + 1 && y0 <= P.b - 1 && y0 + S::TY - 1 >= P.a + 1;
-
   if (tid == 0) {
     for (int s = 0; s < S::RING; ++s) {
       mbar_init(&bar[s], 1);
-      mbar_init(&emp[s], STEP_CONSUMERS / 32);
+      mbar_init(&emp[s], NT / 32);
     }
     mbar_fence_init();
     tma_prefetch_desc(&L.cur);
@@ -122,10 +129,20 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
     tma_prefetch_desc(&L.s);
     tma_prefetch_desc(&L.q);
   }
+  pdl_launch_dependents();
+  pdl_wait();
+  if (!ADJ) sample_detectors(P, ct, tid, (P.n + TW - 1) / TW, (P.n + TH - 1) / TH, NT);
+
+  const int x0 = ct.tx * S::TX, y0 = ct.ty * S::TY;
+  const int k0 = ct.k0;
+  if (k0 >= n) return;  // uniform per CTA
+  const int k1 = min(ct.k1, n);
+  const bool tile_fem = x0 <= P.b - 1 && x0 + S::TX - 1 >= P.a + 1 && y0 <= P.b - 1 && y0 + S::TY - 1 >= P.a + 1;
+
   __syncthreads();
 
-  if (tid >= STEP_CONSUMERS) {
-    if (tid == STEP_CONSUMERS)
+  if (tid >= NT) {
+    if (tid == NT)
       produce_planes<S>(&L.cur, &L.old, &L.s, &L.q, smem, bar, emp, x0, y0, k0, k1, n, tile_fem, P.a, P.b,
                         P.chan, P.spin_limit, P.err);
     return;
@@ -160,7 +177,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
   // corners first, then the others.
   const bool gauss = tile_fem && !P.ebe_r;
   const int gl0 = P.f0 - 1, gl1 = P.f0 + P.nf - (ADJ ? 1 : 0);
-  const int e = (tid - ((nw * nh + 31) & ~31)) & (STEP_CONSUMERS - 1);
+  const int e0 = tid - ((nw * nh + 31) & ~31), e = e0 < 0 ? e0 + NT : e0;
   const bool extra = gauss && e < 2 * (nw + nh) + 4;
   const bool ecol = e < nh + 1, erow = !ecol && e < nw + nh + 1;  // x = -1; y = -1
   int ex = 0, ey = 0;
@@ -198,7 +215,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
     };
     if (own) put(ci, hi, wzp[0]);
     if (extra) put(eci, ehi, wzp[1]);
-    if (!ADJ) compute_sync();
+    if (!ADJ) compute_sync<NT>();
     double *DX = G + S::DX + pl * S::HN, *DY = G + S::DY + pl * S::HN;
     auto diff = [&](int c, int h, bool dx, bool dy) {
       if (ADJ) {
@@ -211,7 +228,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
     };
     if (own) diff(ci, hi, true, true);
     if (extra) diff(eci, ehi, ex < nw, ey < nh);
-    compute_sync();
+    compute_sync<NT>();
   };
   // divergences of the six tetrahedra of the cube at scratch node h (path
   // orders xyz, xzy, yxz, yzx, zxy, zyx)
@@ -257,7 +274,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
     }
     // a timeout ends the loop for the warp, or where the CTA's warps meet at
     // barriers for all of them (the producer times out on unreleased slots)
-    const bool all = gauss ? compute_all(ok) : __all_sync(0xffffffffu, ok);
+    const bool all = gauss ? compute_all<NT>(ok) : __all_sync(0xffffffffu, ok);
     if (!all) {
       if (!ok && (tid & 31) == 0) atomicOr(P.err, 4);
       break;
@@ -280,7 +297,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
       plane_diffs(b1, pl ^ 1, true);
       if (own) cube_divs(hi, qi, pl);
       if (ecube) cube_divs(ehi, eqi, pl);
-      compute_sync();
+      compute_sync<NT>();
       if (own) {
         const double *D = G + S::DIV + qi;
         G[S::FX + qi] = topx + low_x(D);
@@ -301,7 +318,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
           etop = top_y(D);
         }
       }
-      compute_sync();
+      compute_sync<NT>();
       if (own) {
         g[0] = G[S::FX + qi - 1] - G[S::FX + qi];
         g[1] = G[S::FY + qi - CW] - G[S::FY + qi];
@@ -429,26 +446,57 @@ __global__ void __launch_bounds__(STEP_THREADS, 2) k_step64(const __grid_constan
   }
 }
 
-template <bool ADJ, int NB>
+template <bool ADJ, int NB, int TW, int TH>
 cudaError_t set_smem() {
-  return cudaFuncSetAttribute(k_step64<ADJ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, Stage64::SMEM);
+  return cudaFuncSetAttribute(k_step64<ADJ, NB, TW, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Stage64<TW, TH>::SMEM);
+}
+template <int TW, int TH>
+cudaError_t set_smem_tile() {
+  cudaError_t e;
+  if ((e = set_smem<false, 1, TW, TH>()) || (e = set_smem<true, 1, TW, TH>()) ||
+      (e = set_smem<false, BATCH_MAX, TW, TH>()))
+    return e;
+  return set_smem<true, BATCH_MAX, TW, TH>();
+}
+
+template <bool ADJ, int NB, int TW, int TH>
+void launch_tile(const StepLaunch<double, NB> &L, cudaStream_t s) {
+  const int n = L.p[0].n;
+  const dim3 g = L.items ? dim3((unsigned)L.n_items)
+                         : dim3((n + TW - 1) / TW, (n + TH - 1) / TH, L.zchunks * L.nprob);
+  launch_chained(k_step64<ADJ, NB, TW, TH>, g, Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, TH>::SMEM, s,
+                 L.chained != 0, L);
 }
 
 }  // namespace
 
 cudaError_t prepare_step64_kernels() {
   cudaError_t e;
-  if ((e = set_smem<false, 1>()) != cudaSuccess || (e = set_smem<true, 1>()) != cudaSuccess ||
-      (e = set_smem<false, BATCH_MAX>()) != cudaSuccess || (e = set_smem<true, BATCH_MAX>()) != cudaSuccess)
-    return e;
-  return cudaSuccess;
+  if ((e = set_smem_tile<32, 8>()) || (e = set_smem_tile<14, 9>())) return e;
+  return set_smem_tile<8, 8>();
+}
+
+// The smallest tile that still gives the chip's SMs no more than about four
+// (14 x 9), eight (8 x 8) resident thread blocks each in one-plane items: on
+// small grids the FEM cube's nodes, two to three times as dear as the others,
+// then spread over more SMs.  Two and three planes an item are still better
+// with 14 x 9 tiles than one with 32 x 8.
+Tile64 tile64(int n, int count) {
+  auto items = [&](int w, int h) { return (long long)((n + w - 1) / w) * ((n + h - 1) / h) * n * count; };
+  if (items(8, 8) <= 640) return {8, 8};
+  if (items(14, 9) <= 3 * 640) return {14, 9};
+  return {32, 8};
 }
 
 template <bool ADJ, int NB>
 int launch_step64(const StepLaunch<double, NB> &L, cudaStream_t s) {
-  const dim3 g = L.items ? dim3((unsigned)L.n_items)
-                         : dim3(step_tiles_x(L.p[0].n, false), step_tiles_y(L.p[0].n, false), L.zchunks * L.nprob);
-  k_step64<ADJ, NB><<<g, STEP_THREADS, Stage64::SMEM, s>>>(L);
+  if (L.tile_w == 8)
+    launch_tile<ADJ, NB, 8, 8>(L, s);
+  else if (L.tile_w == 14)
+    launch_tile<ADJ, NB, 14, 9>(L, s);
+  else
+    launch_tile<ADJ, NB, 32, 8>(L, s);
   return 1;
 }
 template int launch_step64<false, 1>(const StepLaunch<double, 1> &, cudaStream_t);

@@ -95,19 +95,9 @@ __device__ __forceinline__ void produce_planes(const CUtensorMap *mcur, const CU
     mbar_wait_bounded(&bar[q % S::RING], (uint32_t)((q / S::RING) & 1), spin);
 }
 
-// Tiles per axis of the launch grid (device side of step_tiles_x / _y).  x
-// tiles of the FP32 step kernel: with n = 32 m + 1 the last column is updated
+// x tiles of the FP32 step kernel: with n = 32 m + 1 the last column is updated
 // by the last of m tiles (k_step_pair's x tail) instead of by a tile of its own.
 __host__ __device__ constexpr int tiles_pair_x(int n) { return n % STEP_TX == 1 ? n / STEP_TX : (n + STEP_TX - 1) / STEP_TX; }
-template <typename T>
-__device__ __forceinline__ int step_tiles_dev_x(int n) {
-  return sizeof(T) == 4 ? tiles_pair_x(n) : (n + STEP_TX - 1) / STEP_TX;
-}
-template <typename T>
-__device__ __forceinline__ int step_tiles_dev_y(int n) {
-  return (n + StepTile<T>::TY - 1) / StepTile<T>::TY;
-}
-
 // Tile of this CTA: (problem of the launch, tile x, tile y) and its planes
 // [k0, k1), from the launch's dispatch order if it has one, else from the 3-D
 // grid (z chunks of kz planes).
@@ -138,15 +128,14 @@ __device__ __forceinline__ CtaTile cta_tile(const LT &L) {
 
 // Forward detector sampling of E^n (read-only in the step kernels): the CTAs
 // that own the bottom planes (k0 = 0) of a tile column, one per column
-// whatever the z chunking, share the 3 n_det values by the first 256 threads'
-// index within the column grid.
+// whatever the z chunking, share the 3 n_det values by their computing
+// threads' index within the gx x gy columns.
 template <typename T>
-__device__ __forceinline__ void sample_detectors(const StepParams<T> &P, const CtaTile &ct, int tid) {
-  if (P.n_det <= 0 || ct.k0 != 0 || tid >= STEP_CONSUMERS) return;
-  const int n = P.n;
-  const int gx = step_tiles_dev_x<T>(n), gy = step_tiles_dev_y<T>(n);
-  const long long nb = (long long)gx * gy * STEP_CONSUMERS;
-  for (long long t = ((long long)ct.tx + (long long)gx * ct.ty) * STEP_CONSUMERS + tid; t < 3LL * P.n_det; t += nb) {
+__device__ __forceinline__ void sample_detectors(const StepParams<T> &P, const CtaTile &ct, int tid, int gx, int gy,
+                                                 int threads) {
+  if (P.n_det <= 0 || ct.k0 != 0 || tid >= threads) return;
+  const long long nb = (long long)gx * gy * threads;
+  for (long long t = ((long long)ct.tx + (long long)gx * ct.ty) * threads + tid; t < 3LL * P.n_det; t += nb) {
     const int d = (int)(t / 3), c = (int)(t - 3LL * d);
     P.trace_n[t] = (double)P.cur[c * P.cs + P.det_node[d]];
   }

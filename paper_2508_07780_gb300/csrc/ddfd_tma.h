@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace ddfd {
@@ -87,6 +88,35 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
+// Programmatic dependent launch: a kernel launched `chained` (launch_chained)
+// may start while the kernel before it in the stream still runs, once every
+// block of that one has called pdl_launch_dependents or ended; pdl_wait then
+// waits until it has completed and its writes are visible, to TMA loads too.
+// Both do nothing in a kernel launched in the ordinary way.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+
+// Launches `kernel`; chained: as a programmatic dependent of the kernel
+// launched before it on `s` (which must be a kernel, not a copy or a memset).
+template <typename Kernel, typename Param>
+inline cudaError_t launch_chained(Kernel kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, bool chained,
+                                  const Param &param) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, param);
 }
 
 }  // namespace ddfd

@@ -49,3 +49,28 @@ def test_fp64_step_at_tile_edges(reference, n, fem):
         if first is not None:  # the depth changes no bit
             assert np.array_equal(out["trace"], first["trace"]) and np.array_equal(out["g_eps"], first["g_eps"])
         first = first or out
+
+
+def test_fp64_tiles_of_small_and_large_launches_agree(reference):
+    """The tile shape goes by the nodes of a launch: one problem of 33^3 nodes runs on
+    small tiles (checked against the oracle above), twelve together on the large ones; the
+    arithmetic per node is the same, so every bit is."""
+    from paper_2508_07780_gb300 import Batch
+    rng = np.random.default_rng(3)
+    ws = [workload("tiny", n=33, fem_n=f, n_steps=60, seed=f, dir_seed=f, det_per_side=3) for f in (31, 20, 9)] * 4
+    kw = [dict(n=33, fem_n=w.fem_n, n_steps=60, precision="fp64", src_dir=w.directions(), det_ij=w.detectors(),
+               absorbing_faces=1 | 2 | 4) for w in ws]
+    b = Batch(kw)
+    for m, w in zip(b.members, ws):
+        m.set_coeffs(*w.model())
+    traces = b.forward()
+    eobs = [t + 1e-3 * rng.standard_normal(t.shape) for t in traces]
+    b.adjoint(eobs)
+    for i in (0, 1, 2, 11):
+        w = ws[i]
+        alone = run_gpu(w, eobs[i], precision="fp64", absorbing_faces=1 | 2 | 4)
+        ge, gs = b.members[i].gradient()
+        assert np.abs(ge).max() > 0
+        assert np.array_equal(alone["trace"], traces[i])
+        assert np.array_equal(alone["g_eps"], ge) and np.array_equal(alone["g_sig"], gs)
+    b.close()
