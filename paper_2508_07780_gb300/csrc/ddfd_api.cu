@@ -71,13 +71,77 @@ void dfree(ddfd_problem *p, void *ptr) {
 // about as many items as the chip holds thread blocks (152 SMs x 2, 3 or 4),
 // down to one plane each; beyond that deeper items save halo planes and the
 // Gauss-law term's extra layer per item.
+// FP32: about three items per resident thread block (152 SMs x 2), two planes
+// an item at least: an item starts with the latency of its first planes, which
+// deep items spread, and a step ends when the last item does, which shallow
+// ones bring forward.  us a step (forward / adjoint) at 2, 3, 4, 6, 8, 10, 16
+// planes: 41^3 5.0, 6.2, 7.6 (forward); 65^3 7.2, 8.9 (forward); 100^3 -, -,
+// 13.9 / 14.8, 13.0 / 16.5, -, 19.0 / 24.3; 161^3 with a 121^3 cube 52.0 / 58.5
+// (8), 51.3 / 58.0 (10), 52.9 / 59.3 (16).
 int default_kz(int n, int fp32, int count, Tile64 tile) {
-  if (fp32) return n >= 128 ? 16 : 8;
-  const long long cols = (long long)((n + tile.w - 1) / tile.w) * ((n + tile.h - 1) / tile.h) * count;
+  const long long tx = fp32 ? step_tiles_x(n) : (n + tile.w - 1) / tile.w;
+  const long long ty = fp32 ? step_tiles_y(n) : (n + tile.h - 1) / tile.h;
+  const long long planes = tx * ty * n * count;
+  if (fp32) return (int)std::min<long long>(std::max<long long>((planes + 911) / 912, 2), 16);
   const long long ctas = 152 * (tile.w == 32 ? 2 : tile.w == 14 ? 3 : 4);
-  return (int)std::min<long long>(std::max<long long>((cols * n + ctas / 2) / ctas, 1), 16);
+  return (int)std::min<long long>(std::max<long long>((planes + ctas / 2) / ctas, 1), 16);
 }
-int default_kz_lean(int n) { return n >= 128 ? 16 : 8; }
+
+size_t history_bytes(const ddfd_config &c, bool pad) {
+  if (c.forward_only) return 0;
+  const int f0 = (c.n - c.fem_n) / 2 + 2, nf = c.fem_n - 4;
+  const size_t n_new = c.fem_kind == DDFD_FEM_MESH ? (size_t)c.mesh_n_new : 0;
+  size_t hp = (size_t)nf;
+  if (pad) hp = (size_t)(f0 + nf - f0 / 4 * 4 + 3) / 4 * 4;
+  size_t hcs = hp * nf * nf + n_new;
+  if (pad) hcs = (hcs + 3) / 4 * 4;
+  const size_t seg = c.n_snapshots > 0 ? ((size_t)c.n_steps + c.n_snapshots - 1) / c.n_snapshots : 0;
+  const size_t levels = seg ? seg + 1 : (size_t)c.n_src * (c.n_steps + 1);
+  return levels * 3 * hcs * (c.precision == DDFD_FP32 ? 4 : 8);
+}
+
+// Padding costs 3 % of the history at the benchmark's sizes; what filled the
+// device without it still fits.
+bool history_fits_padded(size_t padded) {
+  size_t fre = 0, total = 0;
+  if (cudaMemGetInfo(&fre, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return padded + total / 16 <= fre;
+}
+
+// At most a 32nd of the memory that is left, and none under a memory budget.
+int build_source_table(ddfd_problem *p) {
+  p->src_off.assign(p->n_src, 0);
+  long long steps = 0;
+  for (int s = 0; s < p->n_src; ++s) {
+    p->src_off[s] = steps;
+    if (p->oblique[s]) steps += std::min((long long)p->n1[s] + 1, (long long)p->Nt);
+  }
+  const size_t row = (size_t)p->n * p->px * (p->fp32 ? 3 : 1);
+  size_t fre = 0, total = 0;
+  if (steps == 0 || p->cfg.mem_budget > 0) return DDFD_OK;
+  CK(cudaMemGetInfo(&fre, &total));
+  if ((size_t)steps * row * p->esz > fre / 32 || dalloc(p, (size_t)steps * row * p->esz, &p->src_tab)) {
+    p->err.clear();
+    return DDFD_OK;
+  }
+  for (int s = 0; s < p->n_src; ++s) {
+    if (!p->oblique[s]) continue;
+    const int k = (int)std::min((long long)p->n1[s] + 1, (long long)p->Nt);
+    auto fill = [&](auto *tab, auto P) {
+      set_source(P, p, s);
+      launch_source_table(P, k, p->tau, tab + (size_t)p->src_off[s] * row, p->stream);
+      ++p->launches;
+    };
+    if (p->fp32)
+      fill((float *)p->src_tab, base_params<float>(p));
+    else
+      fill((double *)p->src_tab, base_params<double>(p));
+  }
+  return sync_check(p);
+}
 
 std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &ps, int kz, int kz_lean,
                                       int *n_full) {
@@ -124,13 +188,19 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
           if (c2) zf0 = std::min(zf0, p->f0), zf1 = std::max(zf1, p->f0 + p->nf);
         }
     }
-    if (zf0 >= zf1) {  // FP64, or no FEM columns: every column in chunks of kz on the full kernel
-      for (int z0 = 0; z0 < n; z0 += kz) full.push_back({cost(z0, std::min(z0 + kz, n)), (int)q, z0, std::min(z0 + kz, n), false});
+    // chunks of kz planes, the last one the rest: a short item at the end of a
+    // column helps the step to end evenly (201^3: 61 / 67 us a forward / adjoint
+    // step, with even chunks 64 / 67)
+    auto cut = [&](int lo, int hi, bool fem) {
+      for (int z0 = lo; z0 < hi; z0 += kz) full.push_back({cost(z0, std::min(z0 + kz, hi)), (int)q, z0, std::min(z0 + kz, hi), fem});
+    };
+    if (zf0 >= zf1) {  // FP64, or no FEM columns: every column as a full item
+      cut(0, n, false);
       continue;
     }
-    // FEM columns: [zf0, zf1) in chunks of kz on the full kernel; the rest of
-    // them and every other column on the lean one (below)
-    for (int z0 = zf0; z0 < zf1; z0 += kz) full.push_back({cost(z0, std::min(z0 + kz, zf1)), (int)q, z0, std::min(z0 + kz, zf1), true});
+    // FEM columns: [zf0, zf1) as full items; the rest of them and every other
+    // column as lean ones (below)
+    cut(zf0, zf1, true);
     lean.push_back({0, (int)q, zf0, zf1, true});
   }
   auto heavy_first = [](const Slab &l, const Slab &r) { return l.cost > r.cost; };
@@ -206,7 +276,6 @@ int build_items(ddfd_problem *p) {
   CK(cudaMemcpy(p->items, it.data(), it.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
   p->items_kz = p->kz;
   p->n_items = (int)it.size();
-  p->items_nfull = n_full;
   return DDFD_OK;
 }
 
@@ -215,24 +284,6 @@ int enqueue_det_sources(ddfd_problem *p, cudaStream_t s) {
   launch_det_sources(p->res, p->Nt, p->n_det, p->n_src, p->n_unode, p->uptr, p->det_list, p->uij, p->n,
                      p->tau * p->tau, 1.0 / (p->h * p->h * p->h), p->rsrc, s);
   return 1;
-}
-
-int make_fork(StepFork *f) {
-  if (cudaStreamCreateWithFlags(&f->side, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&f->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&f->ev_join, cudaEventDisableTiming) != cudaSuccess) {
-    cudaGetLastError();
-    drop_fork(f);
-    return DDFD_E_CUDA;
-  }
-  return DDFD_OK;
-}
-
-void drop_fork(StepFork *f) {
-  if (f->ev_fork) cudaEventDestroy(f->ev_fork);
-  if (f->ev_join) cudaEventDestroy(f->ev_join);
-  if (f->side) cudaStreamDestroy(f->side);
-  *f = StepFork();
 }
 
 uint32_t faces_at(const ddfd_problem *p, int s, long long step) {
@@ -400,9 +451,9 @@ int enqueue_forward(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
       }
       set_forward_step(P, p, s, st, p->E[ic], p->E[io],
                        (p->nsnap || p->fonly) ? nullptr
-                                              : (T *)p->hist + ((size_t)s * (Nt + 1) + st + 1) * 3 * p->n_free);
+                                              : (T *)p->hist + ((size_t)s * (Nt + 1) + st + 1) * 3 * p->hcs);
       enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic]);
-      *nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p, chained), sm, &p->fork);
+      *nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p, chained), sm);
       enqueue_new_step<T>(p, p->X[ic], p->X[io], false, P, sm, nk);
       chained = true;
       std::swap(ic, io);
@@ -450,7 +501,7 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
     for (int j = nseg - 1; j >= 0; --j) {
       const int n0 = p->nsnap ? j * p->seg : 0;
       const int n1 = p->nsnap ? std::min(n0 + p->seg, Nt) : Nt;
-      const T *hbase;  // E^k of this segment at hbase + (k - n0) * 3 n_free
+      const T *hbase;  // E^k of this segment at hbase + (k - n0) * 3 hcs
       if (p->nsnap) {
         // restore the snapshot of step n0 and replay the segment's forward
         // steps, keeping E on the free nodes for the adjoint steps below
@@ -463,21 +514,21 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
         bool chained = false;
         for (int st = n0; st < n1; ++st) {
           // (the trace is written again with the same values)
-          set_forward_step(F, p, s, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->n_free);
+          set_forward_step(F, p, s, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs);
           enqueue_ebe<T>(p, p->E[fc], false, sm, nk);
-          *nk += launch_forward_step(single_launch(F, p->mE_halo[fc], p->mE_ctr[fo], p, chained), sm, &p->fork);
+          *nk += launch_forward_step(single_launch(F, p->mE_halo[fc], p->mE_ctr[fo], p, chained), sm);
           chained = true;
           std::swap(fc, fo);
         }
         hbase = (const T *)p->hist;
       } else {
-        hbase = (const T *)p->hist + (size_t)s * (Nt + 1) * 3 * p->n_free;
+        hbase = (const T *)p->hist + (size_t)s * (Nt + 1) * 3 * p->hcs;
       }
       bool chained = p->nsnap != 0;  // after the segment's replay, or after memsets
       for (int k = n1; k >= n0 + 1; --k) {
-        set_adjoint_step(P, p, s, k, p->Mu[ic], p->Mu[io], hbase + (size_t)(k - n0) * 3 * p->n_free, Nt);
+        set_adjoint_step(P, p, s, k, p->Mu[ic], p->Mu[io], hbase + (size_t)(k - n0) * 3 * p->hcs, Nt);
         enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic]);
-        *nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p, chained), sm, &p->fork);
+        *nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p, chained), sm);
         enqueue_new_step<T>(p, p->XMu[ic], p->XMu[io], true, P, sm, nk);
         chained = true;
         if (p->hist_fem) {  // literal gradient: swap the Gauss-law term of step k (mu^k is still in Mu[ic])
@@ -933,7 +984,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   p->stream = (cudaStream_t)cfg->stream;
   p->tile = ext ? ext->tile : tile64(p->n, 1);
   p->kz = ext ? ext->kz : cfg->tile_kz ? cfg->tile_kz : default_kz(p->n, p->fp32, 1, p->tile);
-  p->kz_lean = ext ? ext->kz_lean : cfg->tile_kz_lean ? cfg->tile_kz_lean : default_kz_lean(p->n);
+  p->kz_lean = ext ? ext->kz_lean : cfg->tile_kz_lean ? cfg->tile_kz_lean : default_kz(p->n, p->fp32, 1, p->tile);
 
   auto bail = [&](int code) {
     g_create_err = p->err;
@@ -945,7 +996,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
       p->err = "cudaEventCreate failed";
       return bail(DDFD_E_CUDA);
     }
-  if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess || make_fork(&p->fork) ||
+  if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
       prepare_step_kernels() != cudaSuccess || prepare_ebe_kernels() != cudaSuccess) {
     p->err = "stream creation or kernel attribute setup failed";
     return bail(DDFD_E_CUDA);
@@ -969,9 +1020,19 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
     p->seg = (p->Nt + cfg->n_snapshots - 1) / cfg->n_snapshots;
     p->nsnap = (p->Nt + p->seg - 1) / p->seg;
   }
-  const size_t histn = p->fonly ? 0
-                       : p->nsnap ? (size_t)(p->seg + 1) * 3 * p->n_free
-                                  : (size_t)p->n_src * (p->Nt + 1) * 3 * p->n_free;
+  p->hx = p->f0;
+  p->hp = p->nf;
+  if (ext ? ext->pad : history_fits_padded(history_bytes(*cfg, true))) {
+    p->hvec = p->fp32 && cfg->mem_budget == 0;
+    if (p->hvec) {
+      p->hx = p->f0 / 4 * 4;
+      p->hp = (p->f0 + p->nf - p->hx + 3) / 4 * 4;
+    }
+  }
+  p->hnew = (long long)p->hp * p->nf * p->nf;
+  p->hcs = p->hnew + p->n_new;
+  if (p->hvec) p->hcs = (p->hcs + 3) / 4 * 4;
+  const size_t hist_bytes = history_bytes(*cfg, p->hvec);
   if (ext) {
     for (int q = 0; q < 2; ++q) {
       p->E[q] = ext->E[q];
@@ -986,7 +1047,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
     return bail(st);
   }
   if ((st = dalloc_t(p, 1, &p->errflag)) ||
-      (st = dalloc(p, histn * p->esz, &p->hist)) || (st = dalloc_t(p, trn, &p->trace)) ||
+      (st = dalloc(p, hist_bytes, &p->hist)) || (st = dalloc_t(p, trn, &p->trace)) ||
       (st = dalloc_t(p, trn, &p->res)) || (st = dalloc_t(p, trn, &p->eobs_stage)) ||
       (st = dalloc_t(p, 2 * (size_t)p->n_free, &p->gacc)) || (st = dalloc_t(p, 4 * (size_t)p->n_free, &p->coef)) ||
       (st = dalloc_t(p, 4 * (size_t)p->n_free, &p->coef_stage)) ||
@@ -995,7 +1056,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
       (st = dalloc_t(p, 1, &p->flag)) || (st = dalloc_t(p, (size_t)std::max(p->n_det, 1), &p->det_node)) ||
       (st = dalloc_t(p, (size_t)p->n * p->n + 1, &p->det_ptr)) ||
       (st = dalloc_t(p, (size_t)std::max(p->n_det, 1), &p->det_list)) ||
-      (p->fp32 && (st = dalloc_t(p, 2 * (size_t)p->n_free, &p->gpart))))
+      (p->fp32 && (st = dalloc_t(p, 2 * (size_t)p->hcs, &p->gpart))))
     return bail(st);
   // detector nodes: the distinct top nodes that carry detectors, in node order
   std::vector<int> dslot((size_t)p->n * p->n, -1), uptr(1, 0), uij;
@@ -1089,6 +1150,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   st = set_coeffs_impl(p, one.data(), zero.data(), nullptr, nullptr, cudaMemcpyHostToDevice);
   p->cfg.cfl_check = chk;
   if (st) return bail(st);
+  if (!ext && (st = build_source_table(p))) return bail(st);  // (a batch does so after its last member)
   *out = p;
   return DDFD_OK;
 }
@@ -1101,7 +1163,6 @@ void destroy_problem(ddfd_problem *p) {
     if (p->ev[q]) cudaEventDestroy(p->ev[q]);
   drop_graphs(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
-  drop_fork(&p->fork);
   delete p;
 }
 

@@ -67,17 +67,17 @@ int single_trial(ddfd_problem *p, int steps, int kz, int kz_lean, float *ms) {
   int ic = 1, io = 0;
   for (int st = 0; st < steps; ++st) {
     set_forward_step(P, p, 0, st, p->E[ic], p->E[io],
-                     p->fonly ? nullptr : (T *)p->hist + trial_hist_index(p, st) * 3 * p->n_free);
+                     p->fonly ? nullptr : (T *)p->hist + trial_hist_index(p, st) * 3 * p->hcs);
     enqueue_ebe<T>(p, p->E[ic], false, sm, &nk, p->X[ic]);
-    nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p), sm, &p->fork);
+    nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p), sm);
     std::swap(ic, io);
   }
   ic = 1, io = 0;
   for (int k = p->fonly ? 0 : steps; k >= 1; --k) {  // forward_only handles time the forward alone
-    set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io], (const T *)p->hist + trial_hist_index(p, k - 1) * 3 * p->n_free,
+    set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io], (const T *)p->hist + trial_hist_index(p, k - 1) * 3 * p->hcs,
                      steps);
     enqueue_ebe<T>(p, p->Mu[ic], true, sm, &nk, p->XMu[ic]);
-    nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p), sm, &p->fork);
+    nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p), sm);
     std::swap(ic, io);
   }
   CK(cudaGetLastError());
@@ -113,7 +113,7 @@ int batch_trial(ddfd_batch *b, int steps, int kz, int kz_lean, float *ms) {
         b, false, all, b->maps.E_halo[ic], b->maps.E_ctr[io],
         [&](StepParams<T> &P, ddfd_problem *p) {
           set_forward_step(P, p, 0, st, p->E[ic], p->E[io],
-                           p->fonly ? nullptr : (T *)p->hist + trial_hist_index(p, st) * 3 * p->n_free);
+                           p->fonly ? nullptr : (T *)p->hist + trial_hist_index(p, st) * 3 * p->hcs);
         },
         sm, &nk, &b->items_all);
     std::swap(ic, io);
@@ -126,7 +126,7 @@ int batch_trial(ddfd_batch *b, int steps, int kz, int kz_lean, float *ms) {
         b, true, all, b->maps.M_halo[ic], b->maps.M_ctr[io],
         [&](StepParams<T> &P, ddfd_problem *p) {
           set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io],
-                           (const T *)p->hist + trial_hist_index(p, k - 1) * 3 * p->n_free, steps);
+                           (const T *)p->hist + trial_hist_index(p, k - 1) * 3 * p->hcs, steps);
         },
         sm, &nk, &b->items_all);
     std::swap(ic, io);

@@ -51,7 +51,6 @@ int build_batch_items(ddfd_batch *b) {
       b->allocs.push_back(d);
       lt.second->d.push_back(d);
       lt.second->n_items.push_back((int)it.size());
-      lt.second->n_full.push_back(n_full);
       BCK(cudaMemcpy(d, it.data(), it.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
     }
   b->items_kz = b->kz;
@@ -89,7 +88,7 @@ int enqueue_batch_forward(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
       }
     auto fill = [&](StepParams<T> &P, ddfd_problem *p) {
       set_forward_step(P, p, 0, st, p->E[ic], p->E[io],
-                       (p->nsnap || p->fonly) ? nullptr : (T *)p->hist + (size_t)(st + 1) * 3 * p->n_free);
+                       (p->nsnap || p->fonly) ? nullptr : (T *)p->hist + (size_t)(st + 1) * 3 * p->hcs);
     };
     // element-by-element members: their FEM rows of this level first
     for (ddfd_problem *p : b->m) enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic], b->errflag);
@@ -149,7 +148,7 @@ int enqueue_batch_adjoint(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
         launch_groups<T>(
             b, false, ck, b->maps.E_halo[fc], b->maps.E_ctr[fo],
             [&](StepParams<T> &P, ddfd_problem *p) {
-              set_forward_step(P, p, 0, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->n_free);
+              set_forward_step(P, p, 0, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs);
             },
             sm, nk, &b->items_ck, st > n0);
         std::swap(fc, fo);
@@ -159,7 +158,7 @@ int enqueue_batch_adjoint(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
     for (int k = n1; k >= n0 + 1; --k) {
       auto fill = [&](StepParams<T> &P, ddfd_problem *p) {
         const long long hk = p->nsnap ? k - n0 : k;
-        set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io], (const T *)p->hist + (size_t)hk * 3 * p->n_free, Nt);
+        set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io], (const T *)p->hist + (size_t)hk * 3 * p->hcs, Nt);
       };
       for (ddfd_problem *p : b->m) enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic], b->errflag);
       launch_groups<T>(b, true, all, b->maps.M_halo[ic], b->maps.M_ctr[io], fill, sm, nk, &b->items_all, chained);
@@ -331,7 +330,6 @@ void destroy_batch(ddfd_batch *b) {
     if (b->ev[q]) cudaEventDestroy(b->ev[q]);
   drop_batch_graphs(b);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-  drop_fork(&b->fork);
   delete b;
 }
 
@@ -395,7 +393,7 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   const int group = std::min(count, BATCH_MAX);
   b->tile = tile64(b->n, group);
   b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : default_kz(b->n, b->fp32, group, b->tile);
-  b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : default_kz_lean(b->n);
+  b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : default_kz(b->n, b->fp32, group, b->tile);
   auto bail = [&](int code, const std::string &m) {
     ddfd::set_thread_error(m);
     destroy_batch(b);
@@ -403,7 +401,7 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   };
   for (int q = 0; q < 4; ++q)
     if (cudaEventCreate(&b->ev[q]) != cudaSuccess) return bail(DDFD_E_CUDA, "cudaEventCreate failed");
-  if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess || make_fork(&b->fork))
+  if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
     return bail(DDFD_E_CUDA, "stream creation failed");
   const size_t slab = 3 * (size_t)b->cs * b->esz * count;
   bool all_fonly = true;
@@ -429,6 +427,9 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   if (encode_field_maps(&m, &b->maps, b->E, b->Mu, b->kcoef, b->n, b->px, b->fp32, count, b->tile))
     return bail(DDFD_E_CUDA, m);
   const size_t fb = 3 * (size_t)b->cs * b->esz;
+  size_t padded = 0;
+  for (int i = 0; i < count; ++i) padded += history_bytes(cfgs[i], true);
+  const bool pad = history_fits_padded(padded);
   for (int i = 0; i < count; ++i) {
     ddfd_config c = cfgs[i];
     c.stream = cfgs[0].stream;
@@ -443,12 +444,15 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
     ms.kz = b->kz;
     ms.kz_lean = b->kz_lean;
     ms.tile = b->tile;
+    ms.pad = pad;
     ddfd_problem *p = nullptr;
     const int st = create_impl(&c, &ms, &p);
     if (st) return bail(st, "member " + std::to_string(i) + ": " + thread_error());
     b->m.push_back(p);
   }
   if (build_batch_items(b)) return bail(DDFD_E_OOM, b->err);
+  for (ddfd_problem *p : b->m)
+    if (const int st = build_source_table(p)) return bail(st, p->err);
   *out = b;
   return DDFD_OK;
 }

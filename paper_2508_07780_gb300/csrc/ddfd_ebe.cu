@@ -410,22 +410,22 @@ __global__ void k_new_step(const NewStepParams<T> P) {
       nw[c] = cen[c] + (q1 * (cen[c] - od[c]) - q2 * R);
       P.old[c * (long long)P.n_new + e] = nw[c];
     }
-    const long long f = P.f0 + e;
+    const long long f = P.f0 + e, hf = P.h0 + e;
     if (!ADJ) {
       if (P.hist_w)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) P.hist_w[c * P.n_free + f] = nw[c];
+        for (int c = 0; c < 3; ++c) P.hist_w[c * P.hcs + hf] = nw[c];
     } else {
       T ge = T(0), gs = T(0);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const T hv = P.hist_r[c * P.n_free + f];
+        const T hv = P.hist_r[c * P.hcs + hf];
         ge += hv * ((nw[c] - T(2) * cen[c] + od[c]) + P.r2 * sx[c]);
         gs += hv * (nw[c] - od[c]);
       }
       if (sizeof(T) == 4) {
         // FP32 block sums folded into the FP64 accumulators (as in the step kernel)
-        float2 *gp = reinterpret_cast<float2 *>(P.gpart) + f;
+        float2 *gp = reinterpret_cast<float2 *>(P.gpart) + hf;
         float a = (float)ge, b = (float)gs;
         if (!(P.gmode & GM_FIRST)) {
           const float2 prev = *gp;

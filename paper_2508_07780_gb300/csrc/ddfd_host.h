@@ -38,16 +38,11 @@ struct FieldMaps {
 };
 
 // Dispatch orders of a batch's step launches over one member list: per group
-// of BATCH_MAX members, the device table and its count of leading items for
-// the full FP32 step kernel.
+// of BATCH_MAX members, the device table and its length.
 struct ItemTables {
   std::vector<uint32_t *> d;
-  std::vector<int> n_items, n_full;
+  std::vector<int> n_items;
 };
-
-// Creates (destroys) the side stream and the two events of a StepFork.
-int make_fork(ddfd::StepFork *f);
-void drop_fork(ddfd::StepFork *f);
 
 }  // namespace host
 }  // namespace ddfd
@@ -70,6 +65,13 @@ struct ddfd_problem {
   void *E[2] = {nullptr, nullptr}, *Mu[2] = {nullptr, nullptr};
   void *kcoef = nullptr;      // padded full-grid (s, q1, q2), 3 channels
   void *hist = nullptr;       // E on the free nodes: every step, or one replayed segment
+  // layout of one step's history: row pitch, x of column 0, component stride,
+  // index of new node 0 (StepParams::hcs, hx, hp)
+  int hp = 0, hx = 0;
+  bool hvec = false;
+  long long hcs = 0, hnew = 0;
+  void *src_tab = nullptr;    // oblique sources (StepParams::src_tab); source s at src_off[s] steps
+  std::vector<long long> src_off;
   void *hist_fem = nullptr;   // literal gradient: E on the FEM-updated nodes, every step
   // checkpointing (n_snapshots > 0): state snapshots (E^n, E^{n-1}) at the
   // starts of segments of seg steps; the adjoint replays each segment
@@ -120,8 +122,6 @@ struct ddfd_problem {
   int kz_lean = 16;           // z depth of the lean FP32 step kernel's items
   uint32_t *items = nullptr;  // dispatch order of the step launches (heaviest slabs first), for items_kz
   int items_kz = 0, n_items = 0;
-  int items_nfull = 0;        // FP32: leading items for the full step kernel, the rest lean
-  ddfd::StepFork fork;        // side stream of the lean step launches
   int n_part = 256;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   double fwd_ms = 0.0, adj_ms = 0.0;
@@ -168,7 +168,6 @@ struct ddfd_batch {
   // the checkpointing members (their replays)
   ddfd::host::ItemTables items_all, items_ck;
   int items_kz = 0;
-  ddfd::StepFork fork;        // side stream of the lean step launches
   // conjugate gradient work space (FP64, free nodes): 14 vectors, partial
   // sums, the 6 reduced scalars
   double *cg = nullptr;
@@ -186,6 +185,7 @@ struct MemberSlot {
   int slot;
   int kz, kz_lean;  // the batch's tile depths
   Tile64 tile;
+  bool pad;         // pad the history's rows (history_fits_padded)
 };
 
 // Message of the last failing handle-less call in this thread.
@@ -214,23 +214,31 @@ int bfail(ddfd_batch *b, int code, const std::string &m);
 int dalloc(ddfd_problem *p, size_t bytes, void **out);
 void dfree(ddfd_problem *p, void *ptr);
 
-// Default z depths of the step kernels' items (tile_kz = 0, tile_kz_lean = 0)
+// Bytes of E on the free nodes that a handle keeps (0 for forward_only), with
+// rows padded to 16 bytes or not; whether `padded` bytes of it leave room on
+// the device (handles with a memory budget never pad).
+size_t history_bytes(const ddfd_config &c, bool pad);
+bool history_fits_padded(size_t padded);
+// Tabulates the oblique sources of a handle (after its other allocations; left
+// out, and evaluated in the step kernels, where memory is short).
+int build_source_table(ddfd_problem *p);
+
+// Default z depth of the step kernels' items (tile_kz = 0, tile_kz_lean = 0)
 // for `count` problems of n^3 nodes.
 int default_kz(int n, int fp32, int count, Tile64 tile);
-int default_kz_lean(int n);
 
 // Dispatch order of one step launch over the problems `ps` (stacked in that
 // order), in z slabs (one problem's z range over a set of its tile columns,
-// in grid order within the slab).  Full-kernel items first (their count in
-// *n_full).  FP64: every column in z chunks of kz, the slabs sorted by an
+// in grid order within the slab).  Full items first (their count in *n_full).
+// FP64: every column in z chunks of at most kz, the slabs sorted by an
 // estimate of their work, heaviest first (node count, plus twice the FEM rows
 // and once the free nodes they hold), ties in order of creation.  FP32: the
 // columns that meet the FEM cube's interior or the free box, over the z range
-// of those boxes, in chunks of kz; then the lean-kernel items in chunks of
-// kz_lean from z = 0: every other column, and the FEM columns' planes outside
-// their full range.  Both FP32 kernels take the problems in the same order
-// (by their full-kernel work, heaviest first) and each problem's slabs in
-// ascending z, so that they stay near each other in time and share halos.
+// of those boxes, in chunks of at most kz; then the lean items in chunks of at
+// most kz_lean: every other column, and the FEM columns' planes outside their
+// full range.  Both kinds take the problems in the same order (by their full
+// items' work, heaviest first) and each problem's slabs in ascending z, so that
+// tiles sharing halo planes run close together in time.
 std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &ps, int kz, int kz_lean,
                                       int *n_full);
 // (Re)builds p->items for p->kz and p->kz_lean.
@@ -313,7 +321,10 @@ StepParams<T> base_params(const ddfd_problem *p) {
   P.det_slot = p->det_slot;
   P.inv_h3 = 1.0 / (p->h * p->h * p->h);
   P.tau2 = p->tau * p->tau;
-  P.n_free = p->n_free;
+  P.hcs = p->hcs;
+  P.hx = p->hx;
+  P.hp = p->hp;
+  P.hvec = p->hvec;
   P.gacc_e = p->gacc;
   P.gacc_s = p->gacc + p->n_free;
   P.gpart = p->gpart;
@@ -339,6 +350,9 @@ void set_forward_step(StepParams<T> &P, const ddfd_problem *p, int s, int st, co
   P.src_y = (T)(P.src_scale * p->ptab[(size_t)s * p->Nt + st]);
   P.trace_n = p->trace + ((size_t)s * (p->Nt + 1) + st) * p->n_det * 3;
   P.hist_w = hist_w;
+  // (source s of the handle: set_source has set P.oblique)
+  const size_t row = (size_t)p->n * p->px * (p->fp32 ? 3 : 1);
+  P.src_tab = p->src_tab && P.oblique && P.src_on ? (const T *)p->src_tab + (size_t)(p->src_off[s] + st) * row : nullptr;
 }
 
 // Per-step scalars of adjoint step k (mu^k -> mu^{k-1}) of source s.
@@ -367,7 +381,6 @@ StepLaunch<T, 1> single_launch(const StepParams<T> &P, const CUtensorMap &cur, c
   L.zchunks = (p->n + P.kz - 1) / P.kz;
   L.items = P.kz == p->items_kz ? p->items : nullptr;
   L.n_items = p->n_items;
-  L.n_full = p->items_nfull;
   L.tile_w = p->tile.w;
   L.chained = chained;
   L.p[0] = P;
@@ -439,7 +452,8 @@ void enqueue_new_step(ddfd_problem *p, const void *cur, void *old, bool adj, con
   N.old = (T *)old;
   N.xcoef = (const T *)p->xcoef;
   N.r2 = S.r2;
-  N.n_free = p->n_free;
+  N.hcs = p->hcs;
+  N.h0 = p->hnew;
   N.f0 = p->n_free_grid;
   N.hist_w = S.hist_w;
   N.hist_r = S.hist_r;
@@ -472,7 +486,6 @@ void launch_groups(ddfd_batch *b, bool adj, const std::vector<int> &idx, const C
     const bool tab = tables && b->kz == b->items_kz && gi < tables->d.size();
     L.items = tab ? tables->d[gi] : nullptr;
     L.n_items = tab ? tables->n_items[gi] : 0;
-    L.n_full = tab ? tables->n_full[gi] : 0;
     L.tile_w = b->tile.w;
     L.chained = chained || g0 > 0;
     for (int g = 0; g < L.nprob; ++g) {
@@ -485,7 +498,7 @@ void launch_groups(ddfd_batch *b, bool adj, const std::vector<int> &idx, const C
       fill(P, p);
       L.p[g] = P;
     }
-    *nk += adj ? launch_adjoint_step(L, sm, &b->fork) : launch_forward_step(L, sm, &b->fork);
+    *nk += adj ? launch_adjoint_step(L, sm) : launch_forward_step(L, sm);
   }
 }
 

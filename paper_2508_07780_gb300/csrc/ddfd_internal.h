@@ -89,9 +89,17 @@ struct StepParams {
   double inv_h3;         // 1 / h^3
   double tau2;           // tau^2
   // history of E on the free nodes
-  T *hist_w;             // forward: hist[n+1] ([3][n_free]); null: not kept
+  // (layout: [3][hcs], node (x, y, k) at (x - hx) + hp ((y - f0) + nf (k - f0));
+  // FP32, hvec: hx and hp multiples of 4, so that a thread's four nodes are
+  // one 16-byte access, the rows' padding included)
+  T *hist_w;             // forward: hist[n+1]; null: not kept
   const T *hist_r;       // adjoint: hist[k]
-  long long n_free;
+  long long hcs;
+  int hx, hp, hvec;
+  // oblique source of this step, tabulated at creation (null: evaluated in
+  // the kernel): FP32 the three components' flux terms [3][n][px], FP64 the
+  // pulse times src_scale [n][px]
+  const T *src_tab;
   double *gacc_e;        // adjoint: gradient accumulators (FP64)
   double *gacc_s;
   // element-by-element FEM rows (fem_kind = DDFD_FEM_EBE): when ebe_r is set,
@@ -105,7 +113,7 @@ struct StepParams {
   uint32_t spin_limit;   // polls per bounded wait
   int chan;              // first channel of this problem in the launch's tensor maps:
                          // fields at chan..chan+2, coefficients (s, q1, q2) likewise
-  float *gpart;          // FP32 adjoint: (g_eps, g_sig) block sums per free node
+  float *gpart;          // FP32 adjoint: (g_eps, g_sig) block sums per free node, in the history's layout
   int gmode;             // FP32 adjoint: GM_FIRST (block starts: no partial to read),
                          // GM_FOLD (block ends: add to the FP64 accumulators)
 };
@@ -127,23 +135,9 @@ struct StepLaunch {
   // chunks of kz planes
   const uint32_t *items;
   int n_items;
-  // FP32 with a dispatch order: items[0, n_full) hold FEM-cube or free nodes
-  // and run on the full step kernel; the rest are finite-difference z ranges
-  // only and run on the lean one (concurrently, on StepFork's side stream)
-  int n_full;
   int tile_w;  // FP64: width of the tile (Tile64)
   int chained; // the work before this launch in its stream is a kernel: launch as its dependent (launch_chained)
   StepParams<T> p[NB];
-};
-
-// Side stream and fork/join events of a step whose FP32 tiles are split
-// between the full and the lean kernel: the lean launch runs on `side`,
-// ordered after the work queued before the step (ev_fork) and before the work
-// queued after it (ev_join), so that both kernels of one step run side by side,
-// also inside a captured graph.
-struct StepFork {
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 // Tiles per axis of the FP32 step kernels' launch grid (32 x 16 tiles, with
@@ -167,12 +161,11 @@ cudaError_t prepare_step64_kernels();
 template <bool ADJ, int NB>
 int launch_step64(const StepLaunch<double, NB> &L, cudaStream_t s);
 
-// One step: returns the number of kernels launched (1, or 2 when the FP32
-// tiles are split; the lean launch goes to fk->side when fk has one, else to s).
+// One step: returns the number of kernels launched.
 template <typename T, int NB>
-int launch_forward_step(const StepLaunch<T, NB> &L, cudaStream_t s, const StepFork *fk = nullptr);
+int launch_forward_step(const StepLaunch<T, NB> &L, cudaStream_t s);
 template <typename T, int NB>
-int launch_adjoint_step(const StepLaunch<T, NB> &L, cudaStream_t s, const StepFork *fk = nullptr);
+int launch_adjoint_step(const StepLaunch<T, NB> &L, cudaStream_t s);
 
 // Element-by-element FEM apply over an explicit tetrahedral mesh, staged in
 // shared memory block by block.  A block holds up to EBE_RB rows (nearby
@@ -304,8 +297,8 @@ struct NewStepParams {
   T *old;                // [3][n_new] in: E^{n-1} / mu^{k+1}, out: E^{n+1} / mu^{k-1}
   const T *xcoef;        // [3][n_new] (s, q1, q2)
   T r2;
-  long long n_free;      // history / accumulator stride
-  long long f0;          // free-node index of new node 0
+  long long hcs;         // component stride of the history
+  long long h0, f0;      // index of new node 0 in the history (and gpart), among the free nodes
   T *hist_w;
   const T *hist_r;
   double *gacc_e, *gacc_s;
@@ -314,6 +307,12 @@ struct NewStepParams {
 };
 template <typename T>
 void launch_new_step(const NewStepParams<T> &P, bool adj, cudaStream_t s);
+
+// The oblique flux of steps 0 .. steps - 1 over the top face, as the step
+// kernels take it (StepParams::src_tab): out [steps][3][n][px] floats, or
+// [steps][n][px] doubles, from base's pulse and the delays [n][n].
+void launch_source_table(const StepParams<float> &base, int steps, double tau, float *out, cudaStream_t s);
+void launch_source_table(const StepParams<double> &base, int steps, double tau, double *out, cudaStream_t s);
 
 // Small kernels.
 void launch_gather_trace(const void *E, int fp32, long long cs, int n_det, const int *det_node,

@@ -383,7 +383,9 @@ __global__ void __launch_bounds__(Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, T
           if (!P.oblique) {
             R[1] -= P.src_y;
           } else {
-            const double v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width, P.t_n - P.delay[x + n * y]);
+            const double v = P.src_tab ? P.src_tab[x + P.px * y]
+                                       : P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width,
+                                                                   P.t_n - P.delay[x + n * y]);
 #pragma unroll
             for (int c = 0; c < 3; ++c) R[c] -= P.pol[c] * v;
           }
@@ -418,13 +420,13 @@ __global__ void __launch_bounds__(Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, T
         if (!ADJ) {
           if (P.hist_w)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) P.hist_w[c * P.n_free + fi] = cen[c] + t[c];
+            for (int c = 0; c < 3; ++c) P.hist_w[c * P.hcs + fi] = cen[c] + t[c];
         } else {
           // mu^{k-1} - 2 mu^k + mu^{k+1} = t - dv, mu^{k-1} - mu^{k+1} = t + dv
           double ge = 0.0, gs = 0.0;
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const double hv = __ldg(P.hist_r + c * P.n_free + fi);
+            const double hv = __ldg(P.hist_r + c * P.hcs + fi);
             ge += hv * ((t[c] - dv[c]) + sx[c]);
             gs += hv * (t[c] + dv[c]);
           }
