@@ -71,7 +71,7 @@ void dfree(ddfd_problem *p, void *ptr) {
 // about as many items as the chip holds thread blocks (152 SMs x 2, 3 or 4),
 // down to one plane each; beyond that deeper items save halo planes and the
 // Gauss-law term's extra layer per item.
-// FP32: about three items per resident thread block (152 SMs x 2), two planes
+// FP32: two to three items per resident thread block (152 SMs x 2), two planes
 // an item at least: an item starts with the latency of its first planes, which
 // deep items spread, and a step ends when the last item does, which shallow
 // ones bring forward.  us a step (forward / adjoint) at 2, 3, 4, 6, 8, 10, 16
@@ -82,7 +82,7 @@ int default_kz(int n, int fp32, int count, Tile64 tile) {
   const long long tx = fp32 ? step_tiles_x(n) : (n + tile.w - 1) / tile.w;
   const long long ty = fp32 ? step_tiles_y(n) : (n + tile.h - 1) / tile.h;
   const long long planes = tx * ty * n * count;
-  if (fp32) return (int)std::min<long long>(std::max<long long>((planes + 911) / 912, 2), 16);
+  if (fp32) return (int)std::min<long long>(std::max<long long>((planes + 719) / 720, 2), 16);
   const long long ctas = 152 * (tile.w == 32 ? 2 : tile.w == 14 ? 3 : 4);
   return (int)std::min<long long>(std::max<long long>((planes + ctas / 2) / ctas, 1), 16);
 }
@@ -452,7 +452,8 @@ int enqueue_forward(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
       set_forward_step(P, p, s, st, p->E[ic], p->E[io],
                        (p->nsnap || p->fonly) ? nullptr
                                               : (T *)p->hist + ((size_t)s * (Nt + 1) + st + 1) * 3 * p->hcs);
-      enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic]);
+      enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic], nullptr, chained);
+      chained = chained || p->ebe_rows > 0;
       *nk += launch_forward_step(single_launch(P, p->mE_halo[ic], p->mE_ctr[io], p, chained), sm);
       enqueue_new_step<T>(p, p->X[ic], p->X[io], false, P, sm, nk);
       chained = true;
@@ -515,7 +516,8 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
         for (int st = n0; st < n1; ++st) {
           // (the trace is written again with the same values)
           set_forward_step(F, p, s, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs);
-          enqueue_ebe<T>(p, p->E[fc], false, sm, nk);
+          enqueue_ebe<T>(p, p->E[fc], false, sm, nk, nullptr, nullptr, chained);
+          chained = chained || p->ebe_rows > 0;
           *nk += launch_forward_step(single_launch(F, p->mE_halo[fc], p->mE_ctr[fo], p, chained), sm);
           chained = true;
           std::swap(fc, fo);
@@ -527,7 +529,8 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
       bool chained = p->nsnap != 0;  // after the segment's replay, or after memsets
       for (int k = n1; k >= n0 + 1; --k) {
         set_adjoint_step(P, p, s, k, p->Mu[ic], p->Mu[io], hbase + (size_t)(k - n0) * 3 * p->hcs, Nt);
-        enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic]);
+        enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic], nullptr, chained);
+        chained = chained || p->ebe_rows > 0;
         *nk += launch_adjoint_step(single_launch(P, p->mM_halo[ic], p->mM_ctr[io], p, chained), sm);
         enqueue_new_step<T>(p, p->XMu[ic], p->XMu[io], true, P, sm, nk);
         chained = true;

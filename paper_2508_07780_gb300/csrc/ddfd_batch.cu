@@ -91,7 +91,10 @@ int enqueue_batch_forward(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
                        (p->nsnap || p->fonly) ? nullptr : (T *)p->hist + (size_t)(st + 1) * 3 * p->hcs);
     };
     // element-by-element members: their FEM rows of this level first
-    for (ddfd_problem *p : b->m) enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic], b->errflag);
+    for (ddfd_problem *p : b->m) {
+      enqueue_ebe<T>(p, p->E[ic], false, sm, nk, p->X[ic], b->errflag, chained);
+      chained = chained || p->ebe_rows > 0;
+    }
     launch_groups<T>(b, false, all, b->maps.E_halo[ic], b->maps.E_ctr[io], fill, sm, nk, &b->items_all, chained);
     chained = true;
     for (ddfd_problem *p : b->m)
@@ -160,7 +163,10 @@ int enqueue_batch_adjoint(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
         const long long hk = p->nsnap ? k - n0 : k;
         set_adjoint_step(P, p, 0, k, p->Mu[ic], p->Mu[io], (const T *)p->hist + (size_t)hk * 3 * p->hcs, Nt);
       };
-      for (ddfd_problem *p : b->m) enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic], b->errflag);
+      for (ddfd_problem *p : b->m) {
+        enqueue_ebe<T>(p, p->Mu[ic], true, sm, nk, p->XMu[ic], b->errflag, chained);
+        chained = chained || p->ebe_rows > 0;
+      }
       launch_groups<T>(b, true, all, b->maps.M_halo[ic], b->maps.M_ctr[io], fill, sm, nk, &b->items_all, chained);
       chained = true;
       for (ddfd_problem *p : b->m)

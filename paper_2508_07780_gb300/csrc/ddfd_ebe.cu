@@ -15,7 +15,7 @@
 // q = h^2 M^-1 (D^T D mu) for the gradient.
 //
 // Staging: blocks of nearby rows (EbeBlock), double-buffered in shared
-// memory by a persistent CTA per SM.  A block's tets arrive as one bulk copy
+// memory by EBE_CTAS persistent CTAs per SM.  A block's tets arrive as one bulk copy
 // and its nodes' values are gathered once into shared memory.  FP32 forward:
 // one thread per tet forms the tet's terms of its four local rows, sum_b
 // (g_a . g_b) E_b + g_a sum_b g_b . (s_b E_b), and writes them over the
@@ -28,6 +28,8 @@
 // terms over the gradients, their sums -- measured slower, 352 against
 // 339 us on 201^3, and is not used.)
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "ddfd_internal.h"
 #include "ddfd_tma.h"
@@ -77,17 +79,20 @@ __device__ __forceinline__ void ld_node(const double *n, double v[4]) {
   v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
 }
 
-// Starts the copies of block `bi` into stage buffer D: the blob by one bulk
-// copy (thread 0, counted on bar), the node values by per-thread copies.
-template <typename T, bool ADJ>
-__device__ __forceinline__ EbeBlock ebe_issue(const EbeParams<T> &P, int bi, unsigned char *D, uint64_t *bar) {
-  const EbeBlock N = P.blocks[bi];
+// Starts the copies of a block into stage buffer D: the blob by one bulk copy
+// (thread 0, counted on bar; static data, so the first one may precede the end
+// of the kernel before), the node values by per-thread copies.
+template <typename T>
+__device__ __forceinline__ void ebe_issue_blob(const EbeParams<T> &P, const EbeBlock &N, int bi, unsigned char *D, uint64_t *bar) {
   // (test hook: block 0's copy is never started, so its wait runs out)
   if (threadIdx.x == 0 && !(P.test_skip_copy && bi == 0)) {
     fence_proxy_async_smem();  // earlier reads of this buffer (ordered by the last barrier) come first
     mbar_expect_tx(bar, (uint32_t)N.bytes);
     bulk_load(D, P.blob + N.blob, (uint32_t)N.bytes, bar);
   }
+}
+template <typename T, bool ADJ>
+__device__ __forceinline__ void ebe_issue_nodes(const EbeParams<T> &P, const EbeBlock &N, unsigned char *D) {
   T *sN = reinterpret_cast<T *>(D + N.bytes);
   for (int i = threadIdx.x; i < N.nn; i += EBE_THREADS) {
     const int o = P.blk_nodes[N.node0 + i];
@@ -118,11 +123,56 @@ __device__ __forceinline__ EbeBlock ebe_issue(const EbeParams<T> &P, int bi, uns
     if (ADJ) sN[4 * i + 3] = T(1);
   }
   cp_async_commit();
-  return N;
+}
+
+// Kuhn stencil rows of an explicit mesh: the same R (and q) as the gather,
+// from the 15-point block stencil of the uniform Kuhn split, R = (6 v_i -
+// sum of the 6 axis neighbours) + sum_o B_o w_{i+o} with w = s E (forward);
+// adjoint R = (6 mu_i - ...) + s_i sum_o B_o mu_{i+o}, q = sum_o B_o mu_{i+o}.
+// The gather's thread blocks do them while their first copies are in flight
+// (as a launch of their own they took 4 us of a 21 us step of the 81^3 mesh).
+template <typename T, bool ADJ>
+__device__ __forceinline__ void kuhn_rows(const KuhnRowParams<T> &P) {
+  const long long sx = 1, sy = P.px, sz = (long long)P.px * P.n;
+  const long long off[7] = {sx, sy, sz, sx + sy, sx + sz, sy + sz, sx + sy + sz};
+  for (int q = blockIdx.x * EBE_THREADS + threadIdx.x; q < P.n_list; q += gridDim.x * EBE_THREADS) {
+    const int r = P.list[q];
+    const long long o = P.row_node[r];
+    T lap[3], g[3] = {T(0), T(0), T(0)};
+    const T s0 = P.s[o];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const T *f = P.field + c * P.cs;
+      lap[c] = T(6) * f[o] - (((((f[o + sx] + f[o - sx]) + f[o + sy]) + f[o - sy]) + f[o + sz]) + f[o - sz]);
+    }
+    {
+      T w[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) w[d] = (ADJ ? T(1) : s0) * P.field[d * P.cs + o];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) g[c] += P.B[0][3 * c] * w[0] + P.B[0][3 * c + 1] * w[1] + P.B[0][3 * c + 2] * w[2];
+    }
+#pragma unroll
+    for (int b = 0; b < 7; ++b) {
+      const long long up = o + off[b], dn = o - off[b];
+      const T su = ADJ ? T(1) : P.s[up], sd = ADJ ? T(1) : P.s[dn];
+      T w[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) w[d] = su * P.field[d * P.cs + up] + sd * P.field[d * P.cs + dn];
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        g[c] += P.B[b + 1][3 * c] * w[0] + P.B[b + 1][3 * c + 1] * w[1] + P.B[b + 1][3 * c + 2] * w[2];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      P.out_r[c * (long long)P.n_rows + r] = lap[c] + (ADJ ? s0 : T(1)) * g[c];
+      if (ADJ) P.out_q[c * (long long)P.n_rows + r] = g[c];
+    }
+  }
 }
 
 template <typename T, bool ADJ>
-__global__ void __launch_bounds__(EBE_THREADS, 1) k_ebe(const EbeParams<T> P) {
+__global__ void __launch_bounds__(EBE_THREADS, EBE_CTAS) k_ebe(const __grid_constant__ EbeParams<T> P) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ int s_ok;
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm);  // one mbarrier per stage
@@ -138,7 +188,14 @@ __global__ void __launch_bounds__(EBE_THREADS, 1) k_ebe(const EbeParams<T> P) {
   auto stage = [&](int q) { return sm + 128 + (size_t)q * P.stage_bytes; };
   int bi = blockIdx.x;
   EbeBlock B;
-  if (bi < P.n_blocks) B = ebe_issue<T, ADJ>(P, bi, stage(0), &bar[0]);
+  if (bi < P.n_blocks) {
+    B = P.blocks[bi];
+    ebe_issue_blob(P, B, bi, stage(0), &bar[0]);
+  }
+  pdl_launch_dependents();
+  pdl_wait();
+  if (bi < P.n_blocks) ebe_issue_nodes<T, ADJ>(P, B, stage(0));
+  kuhn_rows<T, ADJ>(P.kuhn);
   for (; bi < P.n_blocks; bi += gridDim.x) {
     cp_async_wait_all();
     if (tid == 0) s_ok = mbar_wait_bounded(bar + st, (parity >> st) & 1u, P.spin_limit) ? 1 : 0;
@@ -153,7 +210,11 @@ __global__ void __launch_bounds__(EBE_THREADS, 1) k_ebe(const EbeParams<T> P) {
     }
     parity ^= 1u << st;
     EbeBlock next = B;
-    if (bi + (int)gridDim.x < P.n_blocks) next = ebe_issue<T, ADJ>(P, bi + gridDim.x, stage(st ^ 1), bar + (st ^ 1));
+    if (bi + (int)gridDim.x < P.n_blocks) {
+      next = P.blocks[bi + gridDim.x];
+      ebe_issue_blob(P, next, bi + (int)gridDim.x, stage(st ^ 1), bar + (st ^ 1));
+      ebe_issue_nodes<T, ADJ>(P, next, stage(st ^ 1));
+    }
 
     unsigned char *S = stage(st);
     const T *sG = reinterpret_cast<const T *>(S);
@@ -304,79 +365,19 @@ __global__ void __launch_bounds__(EBE_THREADS, 1) k_ebe(const EbeParams<T> P) {
   }
 }
 
-// Kuhn stencil rows of an explicit mesh: the same R (and q) as the gather,
-// from the 15-point block stencil of the uniform Kuhn split, R = (6 v_i -
-// sum of the 6 axis neighbours) + sum_o B_o w_{i+o} with w = s E (forward);
-// adjoint R = (6 mu_i - ...) + s_i sum_o B_o mu_{i+o}, q = sum_o B_o mu_{i+o}.
-template <typename T, bool ADJ>
-__global__ void k_kuhn_rows(const KuhnRowParams<T> P) {
-  const long long sx = 1, sy = P.px, sz = (long long)P.px * P.n;
-  const long long off[7] = {sx, sy, sz, sx + sy, sx + sz, sy + sz, sx + sy + sz};
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < P.n_list; q += gridDim.x * blockDim.x) {
-    const int r = P.list[q];
-    const long long o = P.row_node[r];
-    T lap[3], g[3] = {T(0), T(0), T(0)};
-    const T s0 = P.s[o];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const T *f = P.field + c * P.cs;
-      lap[c] = T(6) * f[o] - (((((f[o + sx] + f[o - sx]) + f[o + sy]) + f[o - sy]) + f[o + sz]) + f[o - sz]);
-    }
-    {
-      T w[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) w[d] = (ADJ ? T(1) : s0) * P.field[d * P.cs + o];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) g[c] += P.B[0][3 * c] * w[0] + P.B[0][3 * c + 1] * w[1] + P.B[0][3 * c + 2] * w[2];
-    }
-#pragma unroll
-    for (int b = 0; b < 7; ++b) {
-      const long long up = o + off[b], dn = o - off[b];
-      const T su = ADJ ? T(1) : P.s[up], sd = ADJ ? T(1) : P.s[dn];
-      T w[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) w[d] = su * P.field[d * P.cs + up] + sd * P.field[d * P.cs + dn];
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        g[c] += P.B[b + 1][3 * c] * w[0] + P.B[b + 1][3 * c + 1] * w[1] + P.B[b + 1][3 * c + 2] * w[2];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      P.out_r[c * (long long)P.n_rows + r] = lap[c] + (ADJ ? s0 : T(1)) * g[c];
-      if (ADJ) P.out_q[c * (long long)P.n_rows + r] = g[c];
-    }
-  }
-}
+static int g_ebe_ctas = 0;  // EBE_CTAS per SM
 
 template <typename T>
-void launch_kuhn_rows(const KuhnRowParams<T> &P, bool adj, cudaStream_t s) {
-  if (P.n_list <= 0) return;
-  const int blocks = (P.n_list + 255) / 256 < 4096 ? (P.n_list + 255) / 256 : 4096;
-  if (adj)
-    k_kuhn_rows<T, true><<<blocks, 256, 0, s>>>(P);
-  else
-    k_kuhn_rows<T, false><<<blocks, 256, 0, s>>>(P);
-}
-
-template void launch_kuhn_rows<float>(const KuhnRowParams<float> &, bool, cudaStream_t);
-template void launch_kuhn_rows<double>(const KuhnRowParams<double> &, bool, cudaStream_t);
-
-static int g_ebe_ctas = 0;  // one CTA per SM
-
-template <typename T>
-void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s) {
-  if (P.n_blocks <= 0) return;
-  const int ctas = g_ebe_ctas > 0 ? g_ebe_ctas : 1;
-  const int grid = P.n_blocks < ctas ? P.n_blocks : ctas;
+void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s, bool chained) {
+  const int want = std::max(P.n_blocks, (P.kuhn.n_list + EBE_THREADS - 1) / EBE_THREADS);
+  if (want <= 0) return;
+  const int grid = std::min(want, g_ebe_ctas > 0 ? g_ebe_ctas : 1);
   const size_t smem = 128 + 2 * (size_t)P.stage_bytes;
-  if (adj)
-    k_ebe<T, true><<<grid, EBE_THREADS, smem, s>>>(P);
-  else
-    k_ebe<T, false><<<grid, EBE_THREADS, smem, s>>>(P);
+  launch_chained(adj ? k_ebe<T, true> : k_ebe<T, false>, dim3((unsigned)grid), EBE_THREADS, smem, s, chained, P);
 }
 
-template void launch_ebe<float>(const EbeParams<float> &, bool, cudaStream_t);
-template void launch_ebe<double>(const EbeParams<double> &, bool, cudaStream_t);
+template void launch_ebe<float>(const EbeParams<float> &, bool, cudaStream_t, bool);
+template void launch_ebe<double>(const EbeParams<double> &, bool, cudaStream_t, bool);
 
 cudaError_t prepare_ebe_kernels() {
   const int lim = 128 + 2 * EBE_SMEM_BUDGET;
@@ -388,7 +389,7 @@ cudaError_t prepare_ebe_kernels() {
       (e = cudaFuncSetAttribute(k_ebe<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
       (e = cudaFuncSetAttribute(k_ebe<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)))
     return e;
-  g_ebe_ctas = sms > 0 ? sms : 1;
+  g_ebe_ctas = sms > 0 ? EBE_CTAS * sms : 1;
   return cudaSuccess;
 }
 
@@ -397,6 +398,8 @@ cudaError_t prepare_ebe_kernels() {
 // adjoint likewise with its transposed rows, and the free-node bookkeeping.
 template <typename T, bool ADJ>
 __global__ void k_new_step(const NewStepParams<T> P) {
+  pdl_launch_dependents();
+  pdl_wait();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < P.n_new; e += gridDim.x * blockDim.x) {
     const long long row = P.row0 + e;
     const T q1 = P.xcoef[P.n_new + e], q2 = P.xcoef[2 * P.n_new + e];
@@ -450,10 +453,7 @@ template <typename T>
 void launch_new_step(const NewStepParams<T> &P, bool adj, cudaStream_t s) {
   if (P.n_new <= 0) return;
   const int blocks = (P.n_new + 255) / 256 < 4096 ? (P.n_new + 255) / 256 : 4096;
-  if (adj)
-    k_new_step<T, true><<<blocks, 256, 0, s>>>(P);
-  else
-    k_new_step<T, false><<<blocks, 256, 0, s>>>(P);
+  launch_chained(adj ? k_new_step<T, true> : k_new_step<T, false>, dim3((unsigned)blocks), 256, 0, s, true, P);
 }
 
 template void launch_new_step<float>(const NewStepParams<float> &, bool, cudaStream_t);

@@ -67,7 +67,7 @@ void kuhn_stencil_rows(long long n_grid_rows, int n, const int *rptr, const int 
 
 bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const double *tgrad, const int *rptr,
                      const int *itet, const int *iloc, const double *rpos, int esz, EbePack *out, std::string *err,
-                     const unsigned char *use) {
+                     const unsigned char *use, int max_rows, int budget) {
   out->blocks.clear();
   out->blob.clear();
   out->nodes.clear();
@@ -168,7 +168,7 @@ bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const d
       }
       const long long nt = (long long)(bt.size() + newT.size());
       const long long bytes = ebe_block_smem(nt, (long long)(bn.size() + newN.size()), std::max(maxinc, deg), esz);
-      const bool fits = (long long)br.size() < EBE_RB && bytes <= EBE_SMEM_BUDGET && nt < (1 << 14);
+      const bool fits = (long long)br.size() < max_rows && bytes <= budget && nt < (1 << 14);
       if (fits) break;
       if (br.empty()) {
         *err = "FEM row " + std::to_string(r) + " has too many elements for the gather's shared memory";

@@ -52,11 +52,25 @@ int upload_ebe(ddfd_problem *p, long long rows, long long ntet, const std::vecto
     p->ebe_bytes_fwd = nt_used * (16 + 12 * es) + nn_used * 4 * es + grows * 3 * es + kr * 7 * es;
     p->ebe_bytes_adj = nt_used * (16 + 12 * es) + nn_used * 3 * es + grows * 6 * es + kr * 10 * es;
   }
+  // blocks of even size in whole rounds over the resident thread blocks: 39^3
+  // rows in blocks of 128 left most SMs idle in a fourth round
+  long long gathered = 0;
+  for (long long r = 0; r < rows; ++r) gathered += !stencil || use[r];
+  int dev = 0, sms = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const long long ctas = (long long)EBE_CTAS * sms;
+  const long long rounds = std::max(1LL, (gathered + EBE_RB * ctas - 1) / (EBE_RB * ctas));
+  const int max_rows = (int)std::min<long long>(EBE_RB, std::max(16LL, (gathered + rounds * ctas - 1) / (rounds * ctas)));
   EbePack pk;
   std::string m;
-  if (!pack_ebe_blocks(rows, ntet, tnode.data(), tgrad.data(), rptr.data(), itet.data(), iloc.data(), rpos.data(),
-                       (int)p->esz, &pk, &m, stencil ? use.data() : nullptr))
-    return fail(p, DDFD_E_ARG, m);
+  // (a row with more elements than half an SM's shared memory takes: blocks of the larger budget)
+  bool packed = false;
+  for (int budget : {EBE_SMEM_SHARED, EBE_SMEM_BUDGET})
+    if ((packed = pack_ebe_blocks(rows, ntet, tnode.data(), tgrad.data(), rptr.data(), itet.data(), iloc.data(),
+                                  rpos.data(), (int)p->esz, &pk, &m, stencil ? use.data() : nullptr, max_rows, budget)))
+      break;
+  if (!packed) return fail(p, DDFD_E_ARG, m);
   if (!klist.empty()) {
     int st;
     if ((st = dalloc_t(p, klist.size(), &p->kuhn_list))) return st;

@@ -387,10 +387,11 @@ StepLaunch<T, 1> single_launch(const StepParams<T> &P, const CUtensorMap &cur, c
   return L;
 }
 
-// The element-by-element rows of the current level (fem_kind = DDFD_FEM_EBE).
+// The element-by-element rows of the current level (fem_kind = DDFD_FEM_EBE);
+// chained: the work before on `sm` is a kernel.
 template <typename T>
 void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, int64_t *nk,
-                 const void *xfield = nullptr, int *err = nullptr) {
+                 const void *xfield = nullptr, int *err = nullptr, bool chained = false) {
   if (!p->ebe_rows) return;
   EbeParams<T> E;
   E.n_rows = p->ebe_rows;
@@ -405,8 +406,9 @@ void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, 
   E.err = err ? err : p->errflag;
   E.spin_limit = p->test_spin ? p->test_spin : 1u << 22;
   E.test_skip_copy = p->test_fault;
+  E.kuhn.n_list = 0;
   if (p->kuhn_n) {
-    KuhnRowParams<T> K;
+    KuhnRowParams<T> &K = E.kuhn;
     K.n_list = p->kuhn_n;
     K.list = p->kuhn_list;
     K.row_node = p->ebe_row_node;
@@ -420,8 +422,6 @@ void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, 
     K.n_rows = p->ebe_rows;
     for (int o = 0; o < 8; ++o)
       for (int e = 0; e < 9; ++e) K.B[o][e] = (T)p->kuhn_B[o][e];
-    launch_kuhn_rows<T>(K, adj, sm);
-    ++*nk;
   }
   E.field = (const T *)field;
   E.s = (const T *)p->kcoef;
@@ -431,8 +431,8 @@ void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, 
   E.xfield = (const T *)xfield;
   E.xs = (const T *)p->xcoef;
   E.n_new = p->n_new;
-  if (p->ebe_nblocks > 0) {
-    launch_ebe<T>(E, adj, sm);
+  if (p->ebe_nblocks > 0 || p->kuhn_n > 0) {
+    launch_ebe<T>(E, adj, sm, chained);
     ++*nk;
   }
 }

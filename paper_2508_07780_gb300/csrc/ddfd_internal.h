@@ -172,13 +172,16 @@ int launch_adjoint_step(const StepLaunch<T, NB> &L, cudaStream_t s);
 // nodes), every tet incident to them and every node of those tets; one CTA
 // copies the block's tets into shared memory, gathers its nodes' values, and
 // then sums each row over its incident tets from shared memory only.
-constexpr int EBE_RB = 128;                  // rows per block
+constexpr int EBE_RB = 64;                   // rows per block
 constexpr int EBE_TPR = 8;                   // threads per row
 constexpr int EBE_THREADS = EBE_TPR * EBE_RB;
-constexpr int EBE_SMEM_BUDGET = 100 * 1024;  // per block (one of two pipeline stages)
+constexpr int EBE_CTAS = 2;                  // thread blocks per SM: one sums while the other waits (81^3 with
+                                             // a 41^3 cube: 13.3 -> 12.8 ms a pass against one of 128 rows)
+constexpr int EBE_SMEM_BUDGET = 100 * 1024;  // per block (one of two pipeline stages), at most
+constexpr int EBE_SMEM_SHARED = 56 * 1024;   // ... where EBE_CTAS share an SM
 constexpr uint16_t EBE_PAD = 0xFFFF;         // unused incidence slot
 
-// The kernel is persistent (one CTA per SM) and double-buffered: while it
+// The kernel is persistent (EBE_CTAS CTAs per SM) and double-buffered: while it
 // sums one block, the next block's blob arrives by bulk copy and its nodes by
 // per-thread asynchronous copies.
 //
@@ -210,8 +213,10 @@ struct EbePack {
 };
 bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const double *tgrad, const int *rptr,
                      const int *itet, const int *iloc, const double *rpos, int esz, EbePack *out, std::string *err,
-                     const unsigned char *use = nullptr);
-// use (may be NULL: every row): rows with use[r] = 0 are left out of the blocks.
+                     const unsigned char *use = nullptr, int max_rows = EBE_RB, int budget = EBE_SMEM_BUDGET);
+// use (may be NULL: every row): rows with use[r] = 0 are left out of the blocks;
+// max_rows, budget: rows (<= EBE_RB) and bytes of shared memory per block at
+// most.
 
 // Marks the grid rows (the first n_grid_rows rows) whose incident tets are
 // exactly the 24 tets of the uniform Kuhn split around the node: 24 incident
@@ -236,8 +241,6 @@ struct KuhnRowParams {
   int n_rows;
   T B[8][9];                // (D^T D)_{i,i+o} / h, offsets 0, (1,0,0) (0,1,0) (0,0,1) (1,1,0) (1,0,1) (0,1,1) (1,1,1)
 };
-template <typename T>
-void launch_kuhn_rows(const KuhnRowParams<T> &P, bool adj, cudaStream_t s);
 // Shared-memory bytes of a block with nt tets, nn nodes, maxinc incidences.
 long long ebe_block_smem(long long nt, long long nn, long long maxinc, int esz);
 
@@ -265,6 +268,7 @@ struct EbeParams {
   const T *xfield;
   const T *xs;
   int n_new;
+  KuhnRowParams<T> kuhn;    // rows taken from the block stencil, in the same launch (n_list 0: none)
 };
 // Sets the shared-memory limit of the gather kernels (once, before any launch).
 cudaError_t prepare_ebe_kernels();
@@ -280,13 +284,15 @@ void launch_copy_fem_nodes(const T *E, T *dst, int n, int px, long long cs, int 
 template <typename T>
 void launch_grad_literal(const T *Efem, const T *mu, double *gacc, int n, int px, long long cs, int a, int b,
                          double r2, cudaStream_t s);
+// chained: the work before on `s` is a kernel (launch_chained)
 template <typename T>
-void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s);
+void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s, bool chained);
 
 // Update of the new nodes of a refined FEM mesh (their rows are FEM rows
 // computed by k_ebe; interior nodes: no boundary or source terms), with the
 // history writes (forward) or the gradient accumulation (adjoint) of the
-// step kernels.
+// step kernels.  It runs as the programmatic dependent of the step kernel
+// before it.
 template <typename T>
 struct NewStepParams {
   int n_new;
