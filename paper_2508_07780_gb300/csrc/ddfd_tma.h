@@ -103,9 +103,9 @@ __device__ __forceinline__ void pdl_wait() {
 
 // Launches `kernel`; chained: as a programmatic dependent of the kernel
 // launched before it on `s` (which must be a kernel, not a copy or a memset).
-template <typename Kernel, typename Param>
-inline cudaError_t launch_chained(Kernel kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, bool chained,
-                                  const Param &param) {
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, bool chained,
+                                  const A &...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
@@ -116,7 +116,7 @@ inline cudaError_t launch_chained(Kernel kernel, dim3 grid, int threads, size_t 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, param);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 }  // namespace ddfd
