@@ -67,10 +67,12 @@ void dfree(ddfd_problem *p, void *ptr) {
     }
 }
 
-// FP64: the step is bound by the SMs' FP64 units, so a small grid is cut into
-// about as many items as the chip holds thread blocks (152 SMs x 2, 3 or 4),
-// down to one plane each; beyond that deeper items save halo planes and the
-// Gauss-law term's extra layer per item.
+// FP64: the step is bound by the SMs' FP64 units: 8 x 8 tiles (small grids) go
+// plane by plane, the others by about 1300 items, 12 planes each at most: deeper
+// items save halo planes and the Gauss-law term's extra layer per item, but end
+// less evenly.  us a step (forward / adjoint): 51^3 23.8 / 23.7, 27.9 / 30.5 (1,
+// 2 planes); 65^3 38.5 / 37.0, 32.1 / 31.5 (1, 2); 100^3 106 / 112, 103 / 108
+// (4, 6); 161^3 466 / 518, 458 / 510 (8, 12).
 // FP32: two to three items per resident thread block (152 SMs x 2), two planes
 // an item at least: an item starts with the latency of its first planes, which
 // deep items spread, and a step ends when the last item does, which shallow
@@ -83,8 +85,8 @@ int default_kz(int n, int fp32, int count, Tile64 tile) {
   const long long ty = fp32 ? step_tiles_y(n) : (n + tile.h - 1) / tile.h;
   const long long planes = tx * ty * n * count;
   if (fp32) return (int)std::min<long long>(std::max<long long>((planes + 719) / 720, 2), 16);
-  const long long ctas = 152 * (tile.w == 32 ? 2 : tile.w == 14 ? 3 : 4);
-  return (int)std::min<long long>(std::max<long long>((planes + ctas / 2) / ctas, 1), 16);
+  if (tile.w == 8) return 1;
+  return (int)std::min<long long>(std::max<long long>((planes + 650) / 1300, 1), 12);
 }
 
 size_t history_bytes(const ddfd_config &c, bool pad) {
@@ -203,10 +205,7 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
     cut(zf0, zf1, true);
     lean.push_back({0, (int)q, zf0, zf1, true});
   }
-  auto heavy_first = [](const Slab &l, const Slab &r) { return l.cost > r.cost; };
-  if (lean.empty()) {
-    std::stable_sort(full.begin(), full.end(), heavy_first);
-  } else {
+  if (!lean.empty()) {
     // problems by FEM work, heaviest first; both kernels take them in that order, z ascending
     std::vector<long long> pc(ps.size(), 0);
     for (const Slab &sl : full) pc[sl.q] += sl.cost;
@@ -230,6 +229,25 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
         if (sl.fem && !colfem[sl.q][(size_t)tx + (size_t)gx * ty]) continue;
         out.push_back(pack_step_item(tx, ty, sl.z0, sl.z1 - sl.z0, sl.q));
       }
+  if (!f32) {
+    // FP64: every item by itself, dearest first (in FP64 instructions of its
+    // warps: 27 a plane, and 70 a layer of cubes that its tile shares with the FEM
+    // rows), so that the thread blocks with FEM rows spread over the SMs and the
+    // cheap ones end the step
+    auto dear = [&](uint32_t it) {
+      const ddfd_problem *p = ps[it >> 28];
+      const int x0 = (int)(it & 31u) * tw, y0 = (int)((it >> 5) & 127u) * ty_rows, z0 = (int)((it >> 12) & 1023u);
+      const int nz = (int)((it >> 22) & 63u) + 1, w = std::min(tw, n - x0), h = std::min(ty_rows, n - y0);
+      const int warps = (w * h + 31) / 32, halo = (2 * (w + h) + 35) / 32;
+      long long c = 27LL * warps * std::min(nz, n - z0);
+      if (meets((int)(it & 31u), (int)((it >> 5) & 127u), p->a + 1, p->b - 1)) {
+        const long long layers = ov(z0 - 1, z0 + nz, p->a + 1, p->b - 1);
+        c += layers * (40LL * warps + 30LL * halo);
+      }
+      return c;
+    };
+    std::stable_sort(out.begin(), out.end(), [&](uint32_t l, uint32_t r) { return dear(l) > dear(r); });
+  }
   *n_full = (int)out.size();
   // lean items: every node's work is the same, so they go by problem and z
   // chunk (chunks of kz_lean from z = 0), all the chunk's columns together,

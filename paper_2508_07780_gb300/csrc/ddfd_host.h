@@ -230,9 +230,8 @@ int default_kz(int n, int fp32, int count, Tile64 tile);
 // Dispatch order of one step launch over the problems `ps` (stacked in that
 // order), in z slabs (one problem's z range over a set of its tile columns,
 // in grid order within the slab).  Full items first (their count in *n_full).
-// FP64: every column in z chunks of at most kz, the slabs sorted by an
-// estimate of their work, heaviest first (node count, plus twice the FEM rows
-// and once the free nodes they hold), ties in order of creation.  FP32: the
+// FP64: every column in z chunks of at most kz, the items by an estimate of
+// their FP64 instructions, dearest first.  FP32: the
 // columns that meet the FEM cube's interior or the free box, over the z range
 // of those boxes, in chunks of at most kz; then the lean items in chunks of at
 // most kz_lean: every other column, and the FEM columns' planes outside their

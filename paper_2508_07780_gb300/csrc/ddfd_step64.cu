@@ -24,10 +24,10 @@
 //
 // Measured (us a step, forward and adjoint averaged, against the 15-point
 // stencil on full 32 x 8 warps with 8 or 16 planes an item): 161^3 with a
-// 121^3 cube 840 -> 584 (the FP64 instructions alone would take about 425),
-// 41^3 / 21^3 88 -> 29 and 13^3 / 9^3 50 -> 12 on 32 x 8 tiles, 19 and 11 on
-// the small tiles below with each step launched as the last one's programmatic
-// dependent (its barriers and descriptors are set up while that one drains).
+// 121^3 cube 840 -> 484 (the FP64 instructions alone would take about 425),
+// 41^3 / 21^3 88 -> 14, 13^3 / 9^3 50 -> 8.  Each step is launched as the last
+// one's programmatic dependent (its barriers and descriptors are set up while
+// that one drains).
 #include "ddfd_step_common.h"
 
 namespace ddfd {
@@ -39,8 +39,7 @@ constexpr int up128(int b) { return (b + 127) / 128 * 128; }
 // A staged plane: the current level and s with a one-node halo in y and a
 // 16-byte halo in x, the previous level and (q1, q2) without.  Three stages:
 // plane k, plane k + 1, and the next one in flight while a plane's FP64 work
-// runs.  Tiles of 32 x 8 nodes (98 KB with the Gauss-law scratch, 2 CTAs per
-// SM); on small grids of 14 x 9 or 8 x 8 (launch_step64).
+// runs.  Tiles of 14 x 9, 8 x 8 or 32 x 8 nodes (tile64).
 template <int TW, int TH>
 struct Stage64 {
   static constexpr int TX = TW;
@@ -479,15 +478,17 @@ cudaError_t prepare_step64_kernels() {
   return set_smem_tile<8, 8>();
 }
 
-// The smallest tile that still gives the chip's SMs no more than about four
-// (14 x 9), eight (8 x 8) resident thread blocks each in one-plane items: on
-// small grids the FEM cube's nodes, two to three times as dear as the others,
-// then spread over more SMs.  Two and three planes an item are still better
-// with 14 x 9 tiles than one with 32 x 8.
+// 14 x 9 tiles: 126 of 128 lanes, warps of their own for the halo nodes, 3
+// thread blocks per SM.  Small grids take 8 x 8 (41^3 13.8 / 14.0 us a forward /
+// adjoint step against 18.5 / 19.1; 51^3 even): the FEM cube's nodes, three times
+// as dear as the others, then spread over more SMs.  32 x 8, two thread blocks per
+// SM (161^3 with a 121^3 cube 530 / 591 us against 458 / 510; 65^3 85 / 96
+// against 32 / 32), is left for the grids whose 14-node columns the dispatch
+// items cannot count.
 Tile64 tile64(int n, int count) {
-  auto items = [&](int w, int h) { return (long long)((n + w - 1) / w) * ((n + h - 1) / h) * n * count; };
-  if (items(8, 8) <= 640) return {8, 8};
-  if (items(14, 9) <= 3 * 640) return {14, 9};
+  const long long items = (long long)((n + 7) / 8) * ((n + 7) / 8) * n * count;
+  if (items <= 2048) return {8, 8};
+  if (n <= 32 * 14) return {14, 9};
   return {32, 8};
 }
 

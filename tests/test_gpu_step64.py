@@ -53,7 +53,7 @@ def test_fp64_step_at_tile_edges(reference, n, fem):
 
 def test_fp64_tiles_of_small_and_large_launches_agree(reference):
     """The tile shape goes by the nodes of a launch: one problem of 33^3 nodes runs on
-    small tiles (checked against the oracle above), twelve together on the large ones; the
+    8 x 8 tiles (checked against the oracle above), twelve together on 14 x 9; the
     arithmetic per node is the same, so every bit is."""
     from paper_2508_07780_gb300 import Batch
     rng = np.random.default_rng(3)
@@ -74,3 +74,28 @@ def test_fp64_tiles_of_small_and_large_launches_agree(reference):
         assert np.array_equal(alone["trace"], traces[i])
         assert np.array_equal(alone["g_eps"], ge) and np.array_equal(alone["g_sig"], gs)
     b.close()
+
+
+def test_fp64_tiles_of_large_grids_against_fp32():
+    """Grids beyond 448 nodes run on 32 x 8 tiles.  Ten steps of a 450^3 grid whose FEM
+    rows reach to two nodes below the top face, against the FP32 kernel, whose rows are
+    written as block stencils: 1e-5 covers its rounding (1e-7 a step) several times over."""
+    from paper_2508_07780_gb300 import Problem, build
+    build.build()
+    n, fem, nt = 450, 448, 10
+    nf = fem - 4
+    z = np.arange(nf)
+    eps = np.broadcast_to((4.0 + 3.0 * ((z // 5) % 3))[:, None, None] + ((z // 7) % 2)[None, None, :], (nf, nf, nf)).ravel()
+    sig = np.broadcast_to((0.1 * ((z // 3) % 4))[None, :, None], (nf, nf, nf)).ravel()
+    det = [[0, 0], [449, 449], [31, 8], [32, 7], [447, 225], [448, 16]]
+    out = {}
+    for prec in ("fp64", "fp32"):
+        p = Problem(n=n, fem_n=fem, n_steps=nt, precision=prec, det_ij=det, freq=2.0, t0=0.05, width=0.5,
+                    src_dir=[[0.3, -0.2, -0.9]])
+        p.set_coeffs(eps, sig)
+        tr = p.forward()
+        p.adjoint(0.5 * tr + 1e-3)
+        out[prec] = (tr, *p.gradient())
+        p.close()
+    for a, b in zip(out["fp64"], out["fp32"]):
+        assert np.abs(a).max() > 0 and rel_l2(b, a) <= 1e-5
