@@ -23,13 +23,14 @@
 // first planes of an item and the last items of a step -- and the instructions of
 // the FEM rows.  us a step, forward / adjoint, against two launches side by side
 // (two nodes a thread, a kernel for the FEM items and one for the others):
-// 201^3 / 101^3 66 / 71 -> 60 / 64, 301^3 / 151^3 190 / 197 -> 183 / 193,
-// 16 x 161^3 (oblique) 597 / 650 -> 573 / 581, 100^3 / 63^3 18 / 19 -> 13.7 / 13.8,
+// 201^3 / 101^3 66 / 71 -> 59 / 64, 301^3 / 151^3 190 / 197 -> 182 / 193,
+// 16 x 161^3 (oblique) 597 / 650 -> 545 / 578, 100^3 / 63^3 18 / 19 -> 13.0 / 13.4,
 // 41^3 / 21^3 10.5 / 11.5 -> 5.1 / 5.0.  Tried and dropped: the last warp to
 // release a slot staging the next plane instead of a producer warp (301^3
 // without a cube 156 -> 180), two nodes a thread (173), carrying the stencil's
 // lower plane in registers (no gain), s = eps - 1 held for all three components
-// (spills).
+// (spills), full and lean items mixed by problem and z (batch 583 -> 642: the two
+// loops share the instruction cache badly).
 //
 // Per node and step:
 //   FD part (every node): 7-point Laplacian with ghost-node (mirror) Neumann
@@ -362,7 +363,11 @@ __device__ __forceinline__ Quad update(const Quad &cen, const Quad &od, const Qu
   return add4(cen, add4(fma4(od, kM1, cen), Q));
 }
 
-template <bool ADJ, int NB>
+// GEN: the launch may hold problems with element-gather rows, unpadded history
+// rows or an oblique source without a table; without it, that code is left out
+// (it crowds registers and the instruction cache: 16 x 161^3 583 -> 545 us a
+// forward step, 587 -> 578 an adjoint one).
+template <bool ADJ, int NB, bool GEN>
 __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_constant__ StepLaunch<float, NB> L) {
   using S = QuadStage;
   constexpr int RE = S::RE, BW = S::BXW, TXY = S::TXY;
@@ -439,7 +444,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
     if (!ADJ && P.src_on) {
       if (!P.oblique) {
         Rn[1] -= P.src_y;
-      } else if (P.src_tab) {
+      } else if (!GEN || P.src_tab) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) Rn[c] -= P.src_tab[xn + P.px * (y + n * c)];
       } else {
@@ -473,7 +478,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
       }
     }
     if (k == n - 1) {
-      if (!ADJ && P.src_on && P.src_tab) {
+      if (!ADJ && P.src_on && (GEN ? P.src_tab != nullptr : P.oblique != 0)) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) Q[c] = add4(Q[c], ld4(P.src_tab + x + P.px * (y + n * c)));
       } else if (ADJ || P.src_on) {
@@ -632,7 +637,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
 #pragma unroll
         for (int c = 0; c < 3; ++c) hv[c] = {kZero, kZero};
         gp[0] = gp[1] = {kZero, kZero};
-        if (P.hvec) {
+        if (!GEN || P.hvec) {
           if (fre) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) hv[c] = ld4(hr + c * P.hcs);
@@ -660,7 +665,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
       // for each component: 36 registers more would spill), the adjoint at the
       // quad's own
       const float *Sm = Em + S::S_OFF / 4, *S0 = E0 + S::S_OFF / 4, *Sp = Ep + S::S_OFF / 4;
-      bool gauss = fem && !P.ebe_r;
+      bool gauss = fem && !(GEN && P.ebe_r);
       Quad sc;
       if (ADJ && gauss) {
         sc = ld4(S0);
@@ -707,7 +712,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
               if (fem) {
                 A = ld4(C0 + S::Q_OFF / 4);
                 C = ld4(C0 + S::Q_OFF / 4 + TXY);
-                if (P.ebe_r) {
+                if (GEN && P.ebe_r) {
                   // element-by-element rows computed by k_ebe for this step
                   const int fm = P.b - P.a - 1;
                   const long long row = (x - P.a - 1) + (long long)fm * ((y - P.a - 1) + (long long)fm * (k - P.a - 1));
@@ -748,7 +753,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
         if (!ADJ) {
           if (P.hist_w) {
             float *hw = P.hist_w + hq;
-            if (P.hvec) {
+            if (!GEN || P.hvec) {
 #pragma unroll
               for (int c = 0; c < 3; ++c) st4(hw + c * P.hcs, nw[c]);
             } else {
@@ -788,7 +793,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
               }
           } else {
             float *g = P.gpart + 2 * (long long)hq;
-            if (P.hvec) {
+            if (!GEN || P.hvec) {
               st4(g, gp[0]), st4(g + 4, gp[1]);
             } else {
 #pragma unroll
@@ -807,7 +812,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
     ++k;
     return true;
   };
-  if (ADJ) {  // (two copies of the turn spill in the adjoint, one with register moves in the forward)
+  if (ADJ || !GEN) {  // (two copies of the turn spill in the adjoint, one with register moves in the general forward)
 #pragma unroll 1
     while (step(q0, q1, q2)) {
 #pragma unroll
@@ -822,7 +827,10 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
 
 template <bool ADJ, int NB>
 static cudaError_t set_smem_f32() {
-  return cudaFuncSetAttribute(k_step_quad<ADJ, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuadStage::SMEM);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_step_quad<ADJ, NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuadStage::SMEM);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_step_quad<ADJ, NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuadStage::SMEM);
 }
 
 cudaError_t prepare_step_kernels() {
@@ -849,7 +857,13 @@ static int launch_step(const StepLaunch<double, NB> &L, cudaStream_t s) {
 }
 template <bool ADJ, int NB>
 static int launch_step(const StepLaunch<float, NB> &L, cudaStream_t s) {
-  launch_chained(k_step_quad<ADJ, NB>, step_grid(L), QUAD_THREADS, QuadStage::SMEM, s, L.chained != 0, L);
+  bool gen = false;
+  for (int q = 0; q < L.nprob; ++q) {
+    const StepParams<float> &P = L.p[q];
+    gen |= P.ebe_r || !P.hvec || (!ADJ && P.src_on && P.oblique && !P.src_tab);
+  }
+  launch_chained(gen ? k_step_quad<ADJ, NB, true> : k_step_quad<ADJ, NB, false>, step_grid(L), QUAD_THREADS,
+                 QuadStage::SMEM, s, L.chained != 0, L);
   return 1;
 }
 
