@@ -618,25 +618,39 @@ int run_sequence(ddfd_problem *p, bool adj) {
   CK(cudaEventRecord(e0, p->stream));
   CK(cudaGraphLaunch(*ge, p->stream));
   CK(cudaEventRecord(e1, p->stream));
-  CK(cudaEventSynchronize(e1));
-  float ms = 0.0f;
-  CK(cudaEventElapsedTime(&ms, e0, e1));
   p->launches += *gl;
   if (adj) {
-    p->adj_ms = ms;
     p->adj_kernels = (int64_t)p->Nt * p->n_src * (p->nsnap ? 2 : 1);
     if (p->nsnap) p->fwd_steps += (int64_t)p->Nt * p->n_src;  // replayed forward steps
   } else {
-    p->fwd_ms = ms;
     p->fwd_kernels = (int64_t)p->Nt * p->n_src;
     p->fwd_steps += (int64_t)p->Nt * p->n_src;
   }
   return DDFD_OK;
 }
 
-int read_flag(ddfd_problem *p, int *out) {
-  CK(cudaMemcpyAsync(out, p->flag, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+// After a sequence, with what has been queued behind it: waits for the stream,
+// takes the sequence's device time and reports a bounded wait that gave up;
+// *flag receives p->flag (one copy and one wait for both).
+int finish_sequence(ddfd_problem *p, bool adj, int *flag) {
+  int *h = (int *)p->hstat;
+  CK(cudaMemcpyAsync(h, p->errflag, 2 * sizeof(int), cudaMemcpyDeviceToHost, p->stream));
   CK(cudaStreamSynchronize(p->stream));
+  float ms = 0.0f;
+  CK(cudaEventElapsedTime(&ms, p->ev[adj ? 2 : 0], p->ev[adj ? 3 : 1]));
+  (adj ? p->adj_ms : p->fwd_ms) = ms;
+  if (h[0]) {
+    CK(cudaMemsetAsync(p->errflag, 0, sizeof(int), p->stream));
+    return fail(p, DDFD_E_TIMEOUT, "a kernel gave up a bounded wait on its TMA copies");
+  }
+  *flag = h[1];
+  return DDFD_OK;
+}
+
+int read_flag(ddfd_problem *p, int *out) {
+  CK(cudaMemcpyAsync(p->hstat, p->flag, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+  CK(cudaStreamSynchronize(p->stream));
+  *out = *(int *)p->hstat;
   return DDFD_OK;
 }
 
@@ -823,14 +837,12 @@ int forward_impl(ddfd_problem *p, double *trace_out, cudaMemcpyKind kind) {
   ++p->generation;
   int st = run_sequence(p, false);
   if (st) return st;
-  if ((st = check_err(p))) return st;
   const long long cnt = (long long)p->n_src * (p->Nt + 1) * p->n_det * 3;
   CK(cudaMemsetAsync(p->flag, 0, sizeof(int), p->stream));
   launch_nonfinite(p->trace, cnt, p->flag, p->stream);
   if (cnt > 0) ++p->launches;
   int flag = 0;
-  int s2 = read_flag(p, &flag);
-  if (s2) return s2;
+  if ((st = finish_sequence(p, false, &flag))) return st;
   p->state = ST_FORWARD;
   if (flag) return fail(p, DDFD_E_NONFINITE, "non-finite value in the forward trace");
   if (trace_out && cnt > 0)
@@ -853,8 +865,8 @@ int functional_impl(ddfd_problem *p, const double *eobs, double *J, bool host) {
   launch_sum(p->part, p->n_part, p->scal + 1, p->stream);
   launch_sum(p->part + p->n_part, p->n_part, p->scal + 2, p->stream);
   p->launches += 5;
-  double v[3];
-  CK(cudaMemcpyAsync(v, p->scal, sizeof(v), cudaMemcpyDeviceToHost, p->stream));
+  const double *v = p->hstat;
+  CK(cudaMemcpyAsync(p->hstat, p->scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
   int st = sync_check(p);
   if (st) return st;
   const double m = p->mass_free ? 1.0 : p->h * p->h * p->h;  // with per-node masses the sums carry them
@@ -878,11 +890,10 @@ int adjoint_impl(ddfd_problem *p, const double *eobs, bool host) {
   ++p->launches;
   p->launches += enqueue_det_sources(p, p->stream);
   p->state = ST_FORWARD;  // the accumulators are overwritten: no earlier gradient survives a failed run
-  int st = run_sequence(p, true);
+  int st = run_sequence(p, true), flag = 0;
   if (st) return st;
-  if ((st = check_err(p))) return st;
-  const int s2 = sync_check(p);
-  if (s2) return s2;
+  if ((st = finish_sequence(p, true, &flag))) return st;
+  CK(cudaGetLastError());
   p->state = ST_ADJOINT;
   return DDFD_OK;
 }
@@ -911,8 +922,10 @@ int gradient_impl(ddfd_problem *p, double *g_eps, double *g_sig, bool host) {
   if (host) {
     CK(cudaMemcpyAsync(g_eps, ge, p->n_free * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
     CK(cudaMemcpyAsync(g_sig, gs, p->n_free * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
+    return sync_check(p);
   }
-  return sync_check(p);
+  CK(cudaGetLastError());  // (the stream is idle since the flag was read)
+  return DDFD_OK;
 }
 
 }  // namespace host
@@ -1022,6 +1035,11 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
     p->err = "stream creation or kernel attribute setup failed";
     return bail(DDFD_E_CUDA);
   }
+  if (cudaHostAlloc((void **)&p->hstat, 64, cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    p->err = "cudaHostAlloc of the status buffer failed";
+    return bail(DDFD_E_CUDA);
+  }
   KuhnBlocks kb;
   if (!build_kuhn_blocks(&kb, &m)) {
     p->err = m;
@@ -1067,18 +1085,19 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
              (st = dalloc(p, 3 * (size_t)p->cs * p->esz, &p->kcoef))) {
     return bail(st);
   }
-  if ((st = dalloc_t(p, 1, &p->errflag)) ||
+  if ((st = dalloc_t(p, 2, &p->errflag)) ||
       (st = dalloc(p, hist_bytes, &p->hist)) || (st = dalloc_t(p, trn, &p->trace)) ||
       (st = dalloc_t(p, trn, &p->res)) || (st = dalloc_t(p, trn, &p->eobs_stage)) ||
       (st = dalloc_t(p, 2 * (size_t)p->n_free, &p->gacc)) || (st = dalloc_t(p, 4 * (size_t)p->n_free, &p->coef)) ||
       (st = dalloc_t(p, 4 * (size_t)p->n_free, &p->coef_stage)) ||
       (st = dalloc_t(p, 2 * (size_t)p->n_free, &p->gout)) || (st = dalloc_t(p, (size_t)p->Nt + 1, &p->z)) ||
       (st = dalloc_t(p, 2 * (size_t)p->n_part, &p->part)) || (st = dalloc_t(p, 4, &p->scal)) ||
-      (st = dalloc_t(p, 1, &p->flag)) || (st = dalloc_t(p, (size_t)std::max(p->n_det, 1), &p->det_node)) ||
+      (st = dalloc_t(p, (size_t)std::max(p->n_det, 1), &p->det_node)) ||
       (st = dalloc_t(p, (size_t)p->n * p->n + 1, &p->det_ptr)) ||
       (st = dalloc_t(p, (size_t)std::max(p->n_det, 1), &p->det_list)) ||
       (p->fp32 && (st = dalloc_t(p, 2 * (size_t)p->hcs, &p->gpart))))
     return bail(st);
+  p->flag = p->errflag + 1;
   // detector nodes: the distinct top nodes that carry detectors, in node order
   std::vector<int> dslot((size_t)p->n * p->n, -1), uptr(1, 0), uij;
   {
@@ -1149,7 +1168,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   }
   launch_coef_vacuum(p->fp32, p->cs, p->kcoef, p->stream);
   ++p->launches;
-  if (cudaMemsetAsync(p->errflag, 0, sizeof(int), p->stream) ||
+  if (cudaMemsetAsync(p->errflag, 0, 2 * sizeof(int), p->stream) ||
  cudaMemsetAsync(p->E[0], 0, fbytes, p->stream) ||
       cudaMemsetAsync(p->E[1], 0, fbytes, p->stream) ||
       (p->Mu[0] && cudaMemsetAsync(p->Mu[0], 0, fbytes, p->stream)) ||
@@ -1180,6 +1199,7 @@ void destroy_problem(ddfd_problem *p) {
   if (p->stream) cudaStreamSynchronize(p->stream);
   else cudaDeviceSynchronize();
   for (void *v : p->allocs) cudaFree(v);
+  if (p->hstat) cudaFreeHost(p->hstat);
   for (int q = 0; q < 4; ++q)
     if (p->ev[q]) cudaEventDestroy(p->ev[q]);
   drop_graphs(p);

@@ -105,7 +105,8 @@ struct ddfd_problem {
   int *det_slot = nullptr, *uptr = nullptr, *uij = nullptr;
   int n_unode = 0;
   float *rsrc = nullptr;
-  int *errflag = nullptr;     // kernel-side error bits (bounded waits)
+  int *errflag = nullptr;     // kernel-side error bits (bounded waits); flag follows it
+  double *hstat = nullptr;    // pinned host copy of small device results (flags, partial functionals)
 
   // TMA descriptors: [buffer] halo-box (current level) and centre-box (old level)
   CUtensorMap mE_halo[2], mE_ctr[2], mM_halo[2], mM_ctr[2], mS, mQ;
