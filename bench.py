@@ -13,9 +13,9 @@ Prints ONE JSON line (rank 0):
               pass, forward + adjoint), device-resident inputs;
   e2e         the same through the host-pointer entry points, with the
               host<->device copies inside the timed region;
-  roofline    the dominant step (the batched adjoint step: its full kernel
-              for the tiles with FEM-cube or free nodes and its lean kernel
-              for the finite-difference tiles, side by side) against the
+  roofline    the dominant step (the batched adjoint step: one launch, full items
+              for the tiles with FEM-cube or free nodes and lean items
+              for the finite-difference tiles) against the
               measured HBM copy bandwidth, with the forward step and the
               whole pass beside it;
   fp64_plain  the plain FP64 GPU path on the same 16 problems, solved one at a
@@ -549,11 +549,11 @@ def run_batched(args, dev, stream, rank, world, peak):
         "bound": "hbm", "achieved": ab / (adj_avg / 1e3) / 1e9, "peak": peak[0], "unit": "GB/s",
         "frac": ab / (adj_avg / 1e3) / 1e9 / peak[0],
         "traffic": traffic_per_launch("batched_adjoint_full_dram_bytes", "batched_adjoint_lean_dram_bytes"),
-        "kernel": "k_step_pair<adjoint,16>: full kernel (tiles with FEM-cube or free nodes) and lean kernel "
-                  "(finite-difference tiles) side by side; one launch = one adjoint step of all 16 problems",
+        "kernel": "k_step_quad<adjoint,16>: full items (tiles with FEM-cube or free nodes) and lean items "
+                  "(finite-difference tiles) in one launch; one launch = one adjoint step of all 16 problems",
         "algorithmic_bytes_per_launch": ab, "avg_launch_ms": adj_avg,
         "peak_kind": f"{peak[1]} (HBM copy, MEASURED_PEAKS.json hbm_gbs)",
-        "forward": {"kernel": "k_step_pair<forward,16>, full and lean kernels side by side",
+        "forward": {"kernel": "k_step_quad<forward,16>, full and lean items in one launch",
                     "algorithmic_bytes_per_launch": fb,
                     "avg_launch_ms": fwd_avg, "achieved": fb / (fwd_avg / 1e3) / 1e9,
                     "frac": fb / (fwd_avg / 1e3) / 1e9 / peak[0],
@@ -621,7 +621,7 @@ def run_fp64_plain(args, dev, stream, probs, out32, fp64_peak):
     fwd_ms, adj_ms = step_ms[3]
     ach = max(ff / (fwd_ms / 1e3), fa / (adj_ms / 1e3)) / 1e12
     roof = {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s", "frac": ach / fp64_peak,
-            "kernel": "k_step<double> (forward and adjoint, problem 3: FEM cube 121^3)",
+            "kernel": "k_step64 (forward and adjoint, problem 3: FEM cube 121^3)",
             "algorithmic_flops_per_launch": {"forward": ff, "adjoint": fa},
             "avg_launch_ms": {"forward": fwd_ms, "adjoint": adj_ms},
             "peak_kind": "measured in this run: cuBLAS DGEMM 4096^3 (torch.matmul float64), best of 5"}
@@ -697,20 +697,20 @@ def run_single_201(args, dev, stream, peak):
     torch.cuda.empty_cache()
     a = out["fp32"]
     fb, ab = algorithmic_bytes(w.n, w.fem_n, 4)
-    kernel_note = "full and lean kernels side by side"
+    kernel_note = "full and lean items in one launch"
     res = {"workload": describe(w), "gradient": args.grad_variant, "value": w.updates / (a["ms"] / 1e3),
            "unit": UNIT, "ms_per_step": a["ms"], "device_bytes": int(a["bytes"]),
            "e_history": (f"checkpointed: {args.snapshots} state snapshots, each segment replayed"
                          if args.snapshots else "kept in HBM for every step"),
            "roofline": {"bound": "hbm", "peak": peak[0], "unit": "GB/s",
-                        "forward": {"kernel": f"k_step_pair<forward,1>, {kernel_note}", "avg_launch_ms": a["fwd"],
+                        "forward": {"kernel": f"k_step_quad<forward,1>, {kernel_note}", "avg_launch_ms": a["fwd"],
                                     "algorithmic_bytes_per_launch": fb,
                                     "frac": fb / (a["fwd"] / 1e3) / 1e9 / peak[0]}}}
     if args.workload == "c2_fp32_201" and not args.snapshots:
         res["roofline"]["forward"]["traffic"] = traffic_per_launch("single_forward_full_dram_bytes",
                                                                    "single_forward_lean_dram_bytes")
     if not args.snapshots:
-        res["roofline"]["adjoint"] = {"kernel": f"k_step_pair<adjoint,1>, {kernel_note}", "avg_launch_ms": a["adj"],
+        res["roofline"]["adjoint"] = {"kernel": f"k_step_quad<adjoint,1>, {kernel_note}", "avg_launch_ms": a["adj"],
                                       "algorithmic_bytes_per_launch": ab,
                                       "frac": ab / (a["adj"] / 1e3) / 1e9 / peak[0]}
         if args.workload == "c2_fp32_201":
@@ -806,7 +806,7 @@ def run_ebe(args, dev, stream, peak):
                      "value": updates / (ms / 1e3), "unit": UNIT, "ms_per_step": ms, "setup_s": setup_s,
                      "gather_roofline": {
                          "bound": "hbm", "peak": peak[0], "unit": "GB/s",
-                         "kernels": "k_ebe" + (" + k_kuhn_rows" if kind else ""),
+                         "kernels": "k_ebe" + (" (Kuhn rows in the same launch)" if kind else ""),
                          "forward": {"ms": fms, "algorithmic_bytes": fb, "achieved": fb / (fms / 1e3) / 1e9,
                                      "frac": fb / (fms / 1e3) / 1e9 / peak[0]},
                          "adjoint": {"ms": ams, "algorithmic_bytes": ab, "achieved": ab / (ams / 1e3) / 1e9,

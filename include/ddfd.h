@@ -108,11 +108,11 @@ typedef struct {
   int32_t cfl_check;     /* nonzero: estimate the stability bound by power iteration
                             at ddfd_set_coeffs and fail with DDFD_E_CFL above it */
   int64_t mem_budget;    /* device bytes the handle may allocate; 0 = no limit */
-  int32_t tile_kz;       /* z planes per thread block of the full step kernel (FP32 tiles
-                            holding FEM-cube or free nodes; every FP64 tile); tuning:
-                            0 = library default (FP32: 16 for n >= 128, else 8; FP64: 1..16
-                            planes, as many as leave an item for every resident thread
-                            block of the GPU), else 2..n */
+  int32_t tile_kz;       /* z planes per thread block of the step kernel's full items (FP32
+                            tiles holding FEM-cube or free nodes; every FP64 tile); tuning:
+                            0 = library default (FP32 2..16, FP64 1..12 planes: as many
+                            as leave an item for every resident thread block of the
+                            GPU), else 2..n */
   int32_t forward_only;  /* nonzero: keep neither the E history nor snapshots (for
                             data generation); ddfd_adjoint then fails with DDFD_E_STATE */
   /* fem_kind = DDFD_FEM_MESH: the tetrahedra of the FEM cube [a, b]^3, a locally
@@ -136,9 +136,9 @@ typedef struct {
                             literal variant keeps E on every FEM-updated node for every step
                             and takes neither n_snapshots, forward_only, fem_kind other than
                             DDFD_FEM_STENCIL, nor batches. */
-  int32_t tile_kz_lean;  /* z planes per thread block of the lean FP32 step kernel (the
-                            finite-difference-only tiles, run beside the full kernel);
-                            tuning: 0 = library default (16 for n >= 128, else 8), else 2..64 */
+  int32_t tile_kz_lean;  /* z planes per thread block of the FP32 step kernel's lean items
+                            (finite-difference-only tiles, in the same launch as the full
+                            ones); tuning: 0 = library default (as tile_kz), else 2..64 */
 } ddfd_config;
 
 /* Fill *cfg with defaults: cfl 0.3, FP64, stencil FEM, 1 normal-incidence
@@ -280,11 +280,11 @@ int ddfd_test_gather_timeout(ddfd_problem *p, int32_t fault, uint32_t spin_limit
  * launch over nprob problems of n^3 nodes (precision DDFD_FP32 or DDFD_FP64)
  * whose FEM cube spans nodes [a, b] and free box [f0, f0 + nf) on each axis,
  * boxes[4 q .. 4 q + 3] = (a, b, f0, nf) for problem q, with z depths kz (full
- * kernel, FP64 kernel) and kz_lean (lean FP32 kernel).  Each item packs tile x
+ * items, FP64 items) and kz_lean (lean FP32 items).  Each item packs tile x
  * (bits 0-4, 32 nodes a tile), tile y (bits 5-11; 16 rows FP32, 8 FP64, the tile
  * of large FP64 launches; small ones run on smaller tiles in the same order), the
  * first plane z0 (bits 12-21), the plane count minus one (bits 22-27) and the
- * problem (bits 28-31); the first *n_full items run on the full kernel.  Up to
+ * problem (bits 28-31); the first *n_full items are full ones.  Up to
  * cap items are written to items (may be NULL with cap = 0); *n_items gets
  * the count.  DDFD_E_ARG: n outside [7, 1024], nprob outside [1, 16], a depth
  * outside [1, 64], a box outside the grid, or cap too small (with *n_items
@@ -294,10 +294,10 @@ int ddfd_test_step_items(int32_t n, int32_t precision, int32_t nprob, const int3
 
 /* Tile autotuner for the step kernels of one handle.  Times `steps` forward
  * and `steps` adjoint steps (CUDA events on the handle's stream) for each
- * candidate z depth of the full kernel's thread-block tiles (4, 6, 8, 12, 16,
- * 24, 32, up to n), the lean kernel's depth held, and keeps the fastest; in
- * FP32 it then does the same for the lean kernel's depth.  *tile_kz_out (may
- * be NULL) receives the full kernel's depth (ddfd_batch_get_info reports
+ * candidate z depth of the full items (4, 6, 8, 12, 16,
+ * 24, 32, up to n), the lean items' depth held, and keeps the fastest; in
+ * FP32 it then does the same for the lean items' depth.  *tile_kz_out (may
+ * be NULL) receives the full items' depth (ddfd_batch_get_info reports
  * both for a batch).  The trial steps overwrite the fields, so forward
  * and adjoint state are invalidated (run ddfd_forward again).  1 <= steps
  * <= n_steps.  The paper has no counterpart (a GPU tuning aid). */
@@ -351,9 +351,9 @@ int ddfd_batch_autotune(ddfd_batch *b, int32_t steps, int32_t *tile_kz_out);
 /* Bookkeeping of a batch: timing of the last batched forward / adjoint
  * sequences (device time, CUDA events on the batch stream; the step-kernel
  * counts count one per batched step of a group of up to 16 members, which
- * runs one kernel, or in FP32 the full and the lean kernel side by side),
+ * runs one kernel),
  * kernels launched, device bytes of the batch and its members, and the tile
- * depths in use (full kernel, lean kernel). */
+ * depths in use (full items, lean items). */
 typedef struct {
   int32_t count, tile_kz;
   double forward_loop_ms, adjoint_loop_ms;

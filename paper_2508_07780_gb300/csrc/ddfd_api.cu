@@ -206,7 +206,7 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
     lean.push_back({0, (int)q, zf0, zf1, true});
   }
   if (!lean.empty()) {
-    // problems by FEM work, heaviest first; both kernels take them in that order, z ascending
+    // problems by FEM work, heaviest first; full and lean items take them in that order, z ascending
     std::vector<long long> pc(ps.size(), 0);
     for (const Slab &sl : full) pc[sl.q] += sl.cost;
     std::vector<int> rank(ps.size());

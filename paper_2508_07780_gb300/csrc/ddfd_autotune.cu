@@ -1,7 +1,7 @@
 // The tile autotuner (ddfd_autotune, ddfd_batch_autotune): times a few
 // forward and adjoint step launches per candidate z depth of the thread-block
-// tiles with CUDA events and keeps the fastest: first the full kernel's depth
-// (the lean one's fixed), then, in FP32, the lean kernel's depth.  A GPU
+// tiles with CUDA events and keeps the fastest: first the full items' depth
+// (the lean ones' fixed), then, in FP32, the lean items' depth.  A GPU
 // tuning aid; the paper has no counterpart.
 #include "ddfd_host.h"
 
@@ -12,7 +12,7 @@ namespace {
 
 const int kTileKz[] = {4, 6, 8, 12, 16, 24, 32};
 
-// Runs trial(kz, kz_lean, &ms) for every candidate z depth of one kernel
+// Runs trial(kz, kz_lean, &ms) for every candidate z depth of one kind of item
 // (after one untimed warm-up trial), the other's held, and returns the
 // fastest in *kz (lean = false) or *kz_lean (lean = true).
 template <typename Trial>

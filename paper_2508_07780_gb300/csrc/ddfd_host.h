@@ -119,8 +119,8 @@ struct ddfd_problem {
   int64_t generation = 0;     // +1 whenever the coefficients or the forward state change
   int64_t launches = 0, fwd_steps = 0;
   ddfd::Tile64 tile;          // FP64 tile shape
-  int kz = 16;                // z depth of the full step kernel's items (and of the FP64 kernel's)
-  int kz_lean = 16;           // z depth of the lean FP32 step kernel's items
+  int kz = 16;                // z depth of the step kernel's full items (and of the FP64 kernel's)
+  int kz_lean = 16;           // z depth of the FP32 step kernel's lean items
   uint32_t *items = nullptr;  // dispatch order of the step launches (heaviest slabs first), for items_kz
   int items_kz = 0, n_items = 0;
   int n_part = 256;

@@ -9,7 +9,7 @@
 //     n = 32 m + 1 nodes the last tile also updates the column x = n - 1.  An
 //     item without FEM-cube or free nodes takes a loop of its own, without the
 //     block stencil, the gradient or the coefficients.
-//   - FP64: ddfd_step64.cu, 32 x 8 tiles or smaller, every tile on one kernel.
+//   - FP64: ddfd_step64.cu, one node a thread, tiles by grid size, every item alike.
 // The planes of the current field (with a one-node halo in y and a
 // 16-byte-aligned halo in x), the centre tile of the previous level, and (on
 // items that touch the FEM cube) the coefficient planes are staged into

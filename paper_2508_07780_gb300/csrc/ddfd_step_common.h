@@ -31,11 +31,7 @@ __device__ __forceinline__ int face_count(int i, int j, int k, int n, uint32_t a
   return f;
 }
 
-// Warp roles: warps 0..7 compute, warp 8 stages planes.
-constexpr int STEP_CONSUMERS = 256;
-constexpr int STEP_THREADS = STEP_CONSUMERS + 32;
-
-// Stages plane p = kk - (k0 - 1) of the chunk into slot p % RING and arms the
+// FP64 (the FP32 kernel stages its two rings itself): stages plane p = kk - (k0 - 1) of the chunk into slot p % RING and arms the
 // slot's "full" barrier with the byte count: the current level (halo box;
 // mirrored ghost planes at kk = -1 and kk = n), the previous level (centre
 // box, computed planes only) and, on tiles touching the FEM cube, s (halo
@@ -96,7 +92,7 @@ __device__ __forceinline__ void produce_planes(const CUtensorMap *mcur, const CU
 }
 
 // x tiles of the FP32 step kernel: with n = 32 m + 1 the last column is updated
-// by the last of m tiles (k_step_pair's x tail) instead of by a tile of its own.
+// by the last of m tiles (the kernel's x tail) instead of by a tile of its own.
 __host__ __device__ constexpr int tiles_pair_x(int n) { return n % STEP_TX == 1 ? n / STEP_TX : (n + STEP_TX - 1) / STEP_TX; }
 // Tile of this CTA: (problem of the launch, tile x, tile y) and its planes
 // [k0, k1), from the launch's dispatch order if it has one, else from the 3-D
