@@ -6,7 +6,7 @@ mod 4, one hemisphere-drawn incident plane wave each, 1600 time steps, 1024
 detectors), stepped together by the batch calls -- per member
 ddfd_set_coeffs, then ddfd_batch_forward, ddfd_functional per member,
 ddfd_batch_adjoint, ddfd_gradient per member.  Every member keeps its E
-history on the free nodes (about 250 GB of HBM in all).
+history on the free nodes (about 265 GB of HBM in all).
 
 Prints ONE JSON line (rank 0):
   value       grid-point updates/s over all ranks (2 n^3 Nt per problem and
