@@ -110,7 +110,7 @@ typedef struct {
   int64_t mem_budget;    /* device bytes the handle may allocate; 0 = no limit */
   int32_t tile_kz;       /* z planes per thread block of the step kernel's full items (FP32
                             tiles holding FEM-cube or free nodes; every FP64 tile); tuning:
-                            0 = library default (FP32 2..16, FP64 1..12 planes: as many
+                            0 = library default (FP32 2..24, FP64 1..12 planes: as many
                             as leave an item for every resident thread block of the
                             GPU), else 2..n */
   int32_t forward_only;  /* nonzero: keep neither the E history nor snapshots (for

@@ -79,12 +79,19 @@ void dfree(ddfd_problem *p, void *ptr) {
 // ones bring forward.  us a step (forward / adjoint) at 2, 3, 4, 6, 8, 10, 16
 // planes: 41^3 5.0, 6.2, 7.6 (forward); 65^3 7.2, 8.9 (forward); 100^3 -, -,
 // 13.9 / 14.8, 13.0 / 16.5, -, 19.0 / 24.3; 161^3 with a 121^3 cube 52.0 / 58.5
-// (8), 51.3 / 58.0 (10), 52.9 / 59.3 (16).
+// (8), 51.3 / 58.0 (10), 52.9 / 59.3 (16).  Batches of 100 planes and more for
+// each of 720 blocks have so many items that their end is even at 24 planes as
+// well, which save halo planes: 16 x 161^3 544 / 578 (16), 530 / 568 (24),
+// 544 / 582 (32).  One large problem gains nothing: 301^3 182 / 193 and 181 / 194
+// (16, 24), 401^3 380 / 386 and 382 / 389.
 int default_kz(int n, int fp32, int count, Tile64 tile) {
   const long long tx = fp32 ? step_tiles_x(n) : (n + tile.w - 1) / tile.w;
   const long long ty = fp32 ? step_tiles_y(n) : (n + tile.h - 1) / tile.h;
   const long long planes = tx * ty * n * count;
-  if (fp32) return (int)std::min<long long>(std::max<long long>((planes + 719) / 720, 2), 16);
+  if (fp32) {
+    const long long kz = std::max<long long>((planes + 719) / 720, 2);
+    return (int)std::min<long long>(kz, count > 1 && kz >= 100 ? 24 : 16);
+  }
   if (tile.w == 8) return 1;
   return (int)std::min<long long>(std::max<long long>((planes + 650) / 1300, 1), 12);
 }

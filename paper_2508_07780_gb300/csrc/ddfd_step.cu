@@ -24,7 +24,7 @@
 // the FEM rows.  us a step, forward / adjoint, against two launches side by side
 // (two nodes a thread, a kernel for the FEM items and one for the others):
 // 201^3 / 101^3 66 / 71 -> 59 / 64, 301^3 / 151^3 190 / 197 -> 182 / 193,
-// 16 x 161^3 (oblique) 597 / 650 -> 545 / 578, 100^3 / 63^3 18 / 19 -> 13.0 / 13.4,
+// 16 x 161^3 (oblique) 597 / 650 -> 530 / 568, 100^3 / 63^3 18 / 19 -> 13.0 / 13.4,
 // 41^3 / 21^3 10.5 / 11.5 -> 5.1 / 5.0.  Tried and dropped: the last warp to
 // release a slot staging the next plane instead of a producer warp (301^3
 // without a cube 156 -> 180), two nodes a thread (173), carrying the stencil's
