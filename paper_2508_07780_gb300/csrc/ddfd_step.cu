@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
           for (int j = 0; j < 4; ++j) {
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-              if (fre && fnode[j]) set(hv[c], j, __ldg(hr + c * P.hcs + j));
+              if (fre && fnode[j]) set(hv[c], j, hr[c * P.hcs + j]);
             if (sums && fnode[j]) (j & 1 ? gp[j >> 1].h : gp[j >> 1].l) = reinterpret_cast<const float2 *>(g)[j];
           }
         }

@@ -27,7 +27,10 @@
 // 121^3 cube 840 -> 484 (the FP64 instructions alone would take about 425),
 // 41^3 / 21^3 88 -> 14, 13^3 / 9^3 50 -> 8.  Each step is launched as the last
 // one's programmatic dependent (its barriers and descriptors are set up while
-// that one drains).
+// that one drains).  So a step may start while the step that writes its fields or
+// its history (a replayed segment's last one) still runs: what that one writes is
+// read by ordinary loads after the wait, never by the non-coherent path, which is
+// for data that nothing writes while the kernel lives.
 #include "ddfd_step_common.h"
 
 namespace ddfd {
@@ -425,7 +428,7 @@ __global__ void __launch_bounds__(Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, T
           double ge = 0.0, gs = 0.0;
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const double hv = __ldg(P.hist_r + c * P.hcs + fi);
+            const double hv = P.hist_r[c * P.hcs + fi];
             ge += hv * ((t[c] - dv[c]) + sx[c]);
             gs += hv * (t[c] + dv[c]);
           }
