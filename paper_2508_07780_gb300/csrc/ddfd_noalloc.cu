@@ -54,14 +54,16 @@ __device__ __forceinline__ double block_sum(double v) {
 // the block.  What bounds the small sizes is the FP64 unit's latency (64 cycles
 // an instruction and warp, whatever its lanes): the taper's cosine is evaluated
 // only in the rows that it touches, t > ramp = T - dl (inv_dl = 1 / dl; ramp is
-// infinite without a taper), by one warp.  Large sizes are bound by the FP64
+// infinite without a taper), by one warp.  Its phase is formed as (t - T) + dl, whose
+// first difference is exact: t - ramp would carry the rounding of T - dl, an error of
+// 1e-16 T / dl in the phase of a short taper.  Large sizes are bound by the FP64
 // unit's rate (two instructions a value).  us a call, before (a thread block per
 // row, two plain launches) and now: 300 steps x 64 detectors 12.3 -> 8.2 (6.8 of
 // it on the host), 2000 x 1024 57 -> 38, 8 sources of it 337 -> 245.
 template <int GROUP>
 __global__ void __launch_bounds__(kRB) k_misfit_rows(const double *__restrict__ trace, const double *__restrict__ eobs,
-                                                     int n_steps, int n_det, int n_rows, double tau, double ramp,
-                                                     double inv_dl, double *rows) {
+                                                     int n_steps, int n_det, int n_rows, double tau, double T,
+                                                     double dl, double ramp, double inv_dl, double *rows) {
   ddfd::pdl_launch_dependents();
   constexpr int PER = kRB / GROUP;
   const int g = threadIdx.x / GROUP, l = threadIdx.x % GROUP;
@@ -84,8 +86,8 @@ __global__ void __launch_bounds__(kRB) k_misfit_rows(const double *__restrict__ 
     }
     double z = 1.0;
     if (l < 32) {
-      const double t = step * tau;
-      if (t > ramp) z = 0.5 * (1.0 + cospi((t - ramp) * inv_dl));
+      const double t = __dmul_rn((double)step, tau);  // (rounded, as T is: T - T has to be zero)
+      if (t > ramp) z = 0.5 * (1.0 + cospi(((t - T) + dl) * inv_dl));
     }
     double b;
     if (GROUP == 32) {
@@ -214,10 +216,10 @@ extern "C" int ddfd_misfit_noalloc(const double *trace, const double *eobs, int3
   if (n_det <= 341) {  // up to 32 values a lane: a warp per row
     const long long nb = (n_rows + kRB / 32 - 1) / (kRB / 32);
     k_misfit_rows<32><<<(int)(nb < 4096 ? nb : 4096), kRB, 0, s>>>(trace, eobs, n_steps, n_det, (int)n_rows, tau,
-                                                                    ramp, inv_dl, rows);
+                                                                    T, dl, ramp, inv_dl, rows);
   } else {
     k_misfit_rows<kRB><<<(int)(n_rows < 4096 ? n_rows : 4096), kRB, 0, s>>>(trace, eobs, n_steps, n_det, (int)n_rows,
-                                                                            tau, ramp, inv_dl, rows);
+                                                                            tau, T, dl, ramp, inv_dl, rows);
   }
   if (n_rows <= 2048)
     ddfd::launch_chained(k_misfit_total<kRB>, dim3(1), kRB, 0, s, true, (const double *)rows, (int)n_rows, tau, J);
