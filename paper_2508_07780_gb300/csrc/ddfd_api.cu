@@ -96,6 +96,8 @@ int default_kz(int n, int fp32, int count, Tile64 tile) {
   return (int)std::min<long long>(std::max<long long>((planes + 650) / 1300, 1), 12);
 }
 
+bool may_pad(const ddfd_config &c) { return c.precision == DDFD_FP32 && c.mem_budget == 0; }
+
 size_t history_bytes(const ddfd_config &c, bool pad) {
   if (c.forward_only) return 0;
   const int f0 = (c.n - c.fem_n) / 2 + 2, nf = c.fem_n - 4;
@@ -109,8 +111,10 @@ size_t history_bytes(const ddfd_config &c, bool pad) {
   return levels * 3 * hcs * (c.precision == DDFD_FP32 ? 4 : 8);
 }
 
-// Padding costs 3 % of the history at the benchmark's sizes; what filled the
-// device without it still fits.
+// Padding costs 3 % of the history at the benchmark's sizes, up to three times it
+// more for a free box of one node.  This is asked before the rest of a handle
+// is allocated, and that may not fit any more: ddfd_create and ddfd_create_batch then
+// begin again without padding, so that what filled the device without it still does.
 bool history_fits_padded(size_t padded) {
   size_t fre = 0, total = 0;
   if (cudaMemGetInfo(&fre, &total) != cudaSuccess) {
@@ -960,7 +964,11 @@ void ddfd_config_default(ddfd_config *c) {
 
 const char *ddfd_create_error(void) { return g_create_err.c_str(); }
 
-int ddfd_create(const ddfd_config *cfg, ddfd_problem **out) { return create_impl(cfg, nullptr, out); }
+int ddfd_create(const ddfd_config *cfg, ddfd_problem **out) {
+  int st = create_impl(cfg, nullptr, out, true);
+  if (st == DDFD_E_OOM && may_pad(*cfg)) st = create_impl(cfg, nullptr, out, false);
+  return st;
+}
 
 void ddfd_destroy(ddfd_problem *p) {
   if (!p || p->batch) return;  // batch members go with their batch
@@ -972,7 +980,7 @@ void ddfd_destroy(ddfd_problem *p) {
 namespace ddfd {
 namespace host {
 
-int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out) {
+int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out, bool pad) {
   g_create_err.clear();
   if (!cfg || !out) {
     g_create_err = "NULL argument";
@@ -1068,12 +1076,10 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   }
   p->hx = p->f0;
   p->hp = p->nf;
-  if (ext ? ext->pad : history_fits_padded(history_bytes(*cfg, true))) {
-    p->hvec = p->fp32 && cfg->mem_budget == 0;
-    if (p->hvec) {
-      p->hx = p->f0 / 4 * 4;
-      p->hp = (p->f0 + p->nf - p->hx + 3) / 4 * 4;
-    }
+  p->hvec = pad && may_pad(*cfg) && (ext || history_fits_padded(history_bytes(*cfg, true)));
+  if (p->hvec) {
+    p->hx = p->f0 / 4 * 4;
+    p->hp = (p->f0 + p->nf - p->hx + 3) / 4 * 4;
   }
   p->hnew = (long long)p->hp * p->nf * p->nf;
   p->hcs = p->hnew + p->n_new;

@@ -341,9 +341,10 @@ void destroy_batch(ddfd_batch *b) {
 
 }  // namespace
 
-extern "C" {
+namespace {
 
-int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) {
+// pad: members that may pad their history's rows do so where it fits.
+int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool pad) {
   ddfd::set_thread_error("");
   if (!cfgs || !out || count < 1 || count > 256) {
     ddfd::set_thread_error("need 1..256 configurations and an output pointer");
@@ -435,7 +436,7 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
   const size_t fb = 3 * (size_t)b->cs * b->esz;
   size_t padded = 0;
   for (int i = 0; i < count; ++i) padded += history_bytes(cfgs[i], true);
-  const bool pad = history_fits_padded(padded);
+  pad = pad && history_fits_padded(padded);
   for (int i = 0; i < count; ++i) {
     ddfd_config c = cfgs[i];
     c.stream = cfgs[0].stream;
@@ -450,9 +451,8 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
     ms.kz = b->kz;
     ms.kz_lean = b->kz_lean;
     ms.tile = b->tile;
-    ms.pad = pad;
     ddfd_problem *p = nullptr;
-    const int st = create_impl(&c, &ms, &p);
+    const int st = create_impl(&c, &ms, &p, pad);
     if (st) return bail(st, "member " + std::to_string(i) + ": " + thread_error());
     b->m.push_back(p);
   }
@@ -461,6 +461,16 @@ int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) 
     if (const int st = build_source_table(p)) return bail(st, p->err);
   *out = b;
   return DDFD_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) {
+  int st = create_batch(cfgs, count, out, true);
+  if (st == DDFD_E_OOM && std::any_of(cfgs, cfgs + count, may_pad)) st = create_batch(cfgs, count, out, false);
+  return st;
 }
 
 void ddfd_destroy_batch(ddfd_batch *b) {

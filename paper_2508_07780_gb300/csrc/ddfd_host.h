@@ -186,7 +186,6 @@ struct MemberSlot {
   int slot;
   int kz, kz_lean;  // the batch's tile depths
   Tile64 tile;
-  bool pad;         // pad the history's rows (history_fits_padded)
 };
 
 // Message of the last failing handle-less call in this thread.
@@ -215,9 +214,11 @@ int bfail(ddfd_batch *b, int code, const std::string &m);
 int dalloc(ddfd_problem *p, size_t bytes, void **out);
 void dfree(ddfd_problem *p, void *ptr);
 
-// Bytes of E on the free nodes that a handle keeps (0 for forward_only), with
-// rows padded to 16 bytes or not; whether `padded` bytes of it leave room on
-// the device (handles with a memory budget never pad).
+// Whether a handle's history rows may be padded to 16 bytes (FP32 handles without
+// a memory budget); bytes of E on the free nodes that a handle keeps (0 for
+// forward_only), with rows padded or not; whether `padded` bytes of it leave room
+// on the device.
+bool may_pad(const ddfd_config &c);
 size_t history_bytes(const ddfd_config &c, bool pad);
 bool history_fits_padded(size_t padded);
 // Tabulates the oblique sources of a handle (after its other allocations; left
@@ -263,7 +264,7 @@ int validate(const ddfd_config *c, std::string *m);
 int grad_mode(int k, int k_first);
 
 // Single-problem operations (ddfd_api.cu).
-int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out);
+int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out, bool pad);
 void destroy_problem(ddfd_problem *p);
 void drop_graphs(ddfd_problem *p);
 int sync_check(ddfd_problem *p);
