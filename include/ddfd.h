@@ -293,12 +293,14 @@ int ddfd_test_step_items(int32_t n, int32_t precision, int32_t nprob, const int3
                          int32_t kz_lean, uint32_t *items, int64_t cap, int64_t *n_items, int64_t *n_full);
 
 /* Tile autotuner for the step kernels of one handle.  Times `steps` forward
- * and `steps` adjoint steps (CUDA events on the handle's stream) for each
- * candidate z depth of the full items (4, 6, 8, 12, 16,
- * 24, 32, up to n), the lean items' depth held, and keeps the fastest; in
- * FP32 it then does the same for the lean items' depth.  *tile_kz_out (may
- * be NULL) receives the full items' depth (ddfd_batch_get_info reports
- * both for a batch).  The trial steps overwrite the fields, so forward
+ * and `steps` adjoint steps (CUDA events on the handle's stream, launched as a
+ * solve launches them) with the handle's z depth of the full items and with
+ * each candidate (4, 6, 8, 12, 16, 24, 32, up to n), the lean items' depth
+ * held, and keeps the fastest: the handle's own depth, which need not be a
+ * candidate, stays unless a candidate is faster.  In FP32 it then does the same for
+ * the lean items' depth.  *tile_kz_out (may be NULL) receives the fastest candidate
+ * for the full items; ddfd_batch_get_info reports the depths that a batch
+ * keeps.  The trial steps overwrite the fields, so forward
  * and adjoint state are invalidated (run ddfd_forward again).  1 <= steps
  * <= n_steps.  The paper has no counterpart (a GPU tuning aid). */
 int ddfd_autotune(ddfd_problem *p, int32_t steps, int32_t *tile_kz_out);

@@ -128,7 +128,7 @@ def main(argv=None):
     b = Batch([dict(n=n, fem_n=fem_n, n_steps=nt, cfl=cfl, precision="fp32", src_dir=d[None, :], det_ij=det,
                     eps_max=max(100.0, a.eps_max), sig_max=max(100.0, a.sig_max), stream=stream, **extra)
                for d in dirs])
-    kz = b.autotune(steps=4)
+    b.autotune(steps=4)
     # step sizes: the first update moves eps by step0 (RMS over the free box);
     # gamma^0 = 1/alpha^0 keeps the step rule's alpha^1 at the same scale
     _, _, probe = b.cg_run(eobs, e0, s0, max_iter=1, gamma_eps0=1.0, gamma_sig0=1.0, alpha_eps0=0.0,
@@ -141,7 +141,7 @@ def main(argv=None):
     ne, ns = np.linalg.norm(e_true), np.linalg.norm(s_true)
     report["initial_eps_rel_err"] = float(np.linalg.norm(e0 - e_true) / ne)
     report["initial_sig_rel_err"] = float(np.linalg.norm(s0 - s_true) / ns)
-    report["tile_kz"] = kz
+    report["tile_kz"] = b.get_info().tile_kz
     report["updates_per_iteration"] = 2 * n ** 3 * nt * a.sources
     for variant in a.variants.split(","):
         prm = dict(max_iter=a.iters, gamma_eps0=1.0 / alpha_e, gamma_sig0=1.0 / alpha_s, alpha_eps0=alpha_e,
