@@ -110,9 +110,9 @@ typedef struct {
   int64_t mem_budget;    /* device bytes the handle may allocate; 0 = no limit */
   int32_t tile_kz;       /* z planes per thread block of the step kernel's full items (FP32
                             tiles holding FEM-cube or free nodes; every FP64 tile); tuning:
-                            0 = library default (FP32 2..24, FP64 1..12 planes: as many
-                            as leave an item for every resident thread block of the
-                            GPU), else 2..n */
+                            0 = library default (FP32 2..24, FP64 1..12 planes: few enough
+                            that every resident thread block of the GPU has two to three
+                            items), else FP32 2..n, FP64 1..n */
   int32_t forward_only;  /* nonzero: keep neither the E history nor snapshots (for
                             data generation); ddfd_adjoint then fails with DDFD_E_STATE */
   /* fem_kind = DDFD_FEM_MESH: the tetrahedra of the FEM cube [a, b]^3, a locally
@@ -138,7 +138,8 @@ typedef struct {
                             DDFD_FEM_STENCIL, nor batches. */
   int32_t tile_kz_lean;  /* z planes per thread block of the FP32 step kernel's lean items
                             (finite-difference-only tiles, in the same launch as the full
-                            ones); tuning: 0 = library default (as tile_kz), else 2..64 */
+                            ones; not used in FP64); tuning: 0 = library default (as
+                            tile_kz), else FP32 2..64, FP64 1..64 */
 } ddfd_config;
 
 /* Fill *cfg with defaults: cfl 0.3, FP64, stencil FEM, 1 normal-incidence

@@ -363,9 +363,12 @@ int validate(const ddfd_config *c, std::string *m) {
   if (!(c->eps_max >= 1.0) || !(c->sig_max >= 0.0)) return *m = "bad coefficient bounds", DDFD_E_ARG;
   if (c->n_snapshots < 0 || c->n_snapshots > c->n_steps) return *m = "n_snapshots must be in [0, n_steps]", DDFD_E_ARG;
   if (c->mem_budget < 0) return *m = "mem_budget must be >= 0", DDFD_E_ARG;
-  if (c->tile_kz != 0 && (c->tile_kz < 2 || c->tile_kz > c->n)) return *m = "tile_kz must be 0 or in [2, n]", DDFD_E_ARG;
-  if (c->tile_kz_lean != 0 && (c->tile_kz_lean < 2 || c->tile_kz_lean > ITEM_MAX_NZ))
-    return *m = "tile_kz_lean must be 0 or in [2, 64]", DDFD_E_ARG;
+  // (FP64: from 1, the default depth of small grids, which a batch reports)
+  const int kz_min = c->precision == DDFD_FP64 ? 1 : 2;
+  if (c->tile_kz != 0 && (c->tile_kz < kz_min || c->tile_kz > c->n))
+    return *m = "tile_kz must be 0 or in [" + std::to_string(kz_min) + ", n]", DDFD_E_ARG;
+  if (c->tile_kz_lean != 0 && (c->tile_kz_lean < kz_min || c->tile_kz_lean > ITEM_MAX_NZ))
+    return *m = "tile_kz_lean must be 0 or in [" + std::to_string(kz_min) + ", 64]", DDFD_E_ARG;
   if (c->src_dir)
     for (int s = 0; s < c->n_src; ++s) {
       const double *k = c->src_dir + 3 * s;
