@@ -96,6 +96,8 @@ int default_kz(int n, int fp32, int count, Tile64 tile) {
   return (int)std::min<long long>(std::max<long long>((planes + 650) / 1300, 1), 12);
 }
 
+int tight_kz(int n) { return n >= 128 ? 16 : 8; }
+
 bool may_pad(const ddfd_config &c) { return c.precision == DDFD_FP32 && c.mem_budget == 0; }
 
 size_t history_bytes(const ddfd_config &c, bool pad) {
@@ -113,8 +115,8 @@ size_t history_bytes(const ddfd_config &c, bool pad) {
 
 // Padding costs 3 % of the history at the benchmark's sizes, up to three times it
 // more for a free box of one node.  This is asked before the rest of a handle
-// is allocated, and that may not fit any more: ddfd_create and ddfd_create_batch then
-// begin again without padding, so that what filled the device without it still does.
+// is allocated, and that may not fit any more: the handle is then created anew in
+// its tight form (create_impl).
 bool history_fits_padded(size_t padded) {
   size_t fre = 0, total = 0;
   if (cudaMemGetInfo(&fre, &total) != cudaSuccess) {
@@ -968,9 +970,8 @@ void ddfd_config_default(ddfd_config *c) {
 const char *ddfd_create_error(void) { return g_create_err.c_str(); }
 
 int ddfd_create(const ddfd_config *cfg, ddfd_problem **out) {
-  int st = create_impl(cfg, nullptr, out, true);
-  if (st == DDFD_E_OOM && may_pad(*cfg)) st = create_impl(cfg, nullptr, out, false);
-  return st;
+  const int st = create_impl(cfg, nullptr, out, false);
+  return st == DDFD_E_OOM ? create_impl(cfg, nullptr, out, true) : st;
 }
 
 void ddfd_destroy(ddfd_problem *p) {
@@ -983,7 +984,7 @@ void ddfd_destroy(ddfd_problem *p) {
 namespace ddfd {
 namespace host {
 
-int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out, bool pad) {
+int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out, bool tight) {
   g_create_err.clear();
   if (!cfg || !out) {
     g_create_err = "NULL argument";
@@ -1034,9 +1035,11 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   p->fp32 = cfg->precision == DDFD_FP32;
   p->esz = p->fp32 ? 4 : 8;
   p->stream = (cudaStream_t)cfg->stream;
-  p->tile = ext ? ext->tile : tile64(p->n, 1);
-  p->kz = ext ? ext->kz : cfg->tile_kz ? cfg->tile_kz : default_kz(p->n, p->fp32, 1, p->tile);
-  p->kz_lean = ext ? ext->kz_lean : cfg->tile_kz_lean ? cfg->tile_kz_lean : default_kz(p->n, p->fp32, 1, p->tile);
+  p->tight = tight;
+  p->tile = ext ? ext->tile : tight ? Tile64() : tile64(p->n, 1);
+  const int kz = tight ? tight_kz(p->n) : default_kz(p->n, p->fp32, 1, p->tile);
+  p->kz = ext ? ext->kz : cfg->tile_kz ? cfg->tile_kz : kz;
+  p->kz_lean = ext ? ext->kz_lean : cfg->tile_kz_lean ? cfg->tile_kz_lean : kz;
 
   auto bail = [&](int code) {
     g_create_err = p->err;
@@ -1079,7 +1082,7 @@ int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **ou
   }
   p->hx = p->f0;
   p->hp = p->nf;
-  p->hvec = pad && may_pad(*cfg) && (ext || history_fits_padded(history_bytes(*cfg, true)));
+  p->hvec = !tight && may_pad(*cfg) && (ext ? ext->pad : history_fits_padded(history_bytes(*cfg, true)));
   if (p->hvec) {
     p->hx = p->f0 / 4 * 4;
     p->hp = (p->f0 + p->nf - p->hx + 3) / 4 * 4;

@@ -343,8 +343,8 @@ void destroy_batch(ddfd_batch *b) {
 
 namespace {
 
-// pad: members that may pad their history's rows do so where it fits.
-int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool pad) {
+// tight: every member in its tight form (create_impl).
+int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool tight) {
   ddfd::set_thread_error("");
   if (!cfgs || !out || count < 1 || count > 256) {
     ddfd::set_thread_error("need 1..256 configurations and an output pointer");
@@ -398,9 +398,10 @@ int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool 
   b->seg = seg;
   b->stream = (cudaStream_t)cfgs[0].stream;
   const int group = std::min(count, BATCH_MAX);
-  b->tile = tile64(b->n, group);
-  b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : default_kz(b->n, b->fp32, group, b->tile);
-  b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : default_kz(b->n, b->fp32, group, b->tile);
+  b->tile = tight ? Tile64() : tile64(b->n, group);
+  const int kz = tight ? tight_kz(b->n) : default_kz(b->n, b->fp32, group, b->tile);
+  b->kz = cfgs[0].tile_kz ? cfgs[0].tile_kz : kz;
+  b->kz_lean = cfgs[0].tile_kz_lean ? cfgs[0].tile_kz_lean : kz;
   auto bail = [&](int code, const std::string &m) {
     ddfd::set_thread_error(m);
     destroy_batch(b);
@@ -436,7 +437,7 @@ int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool 
   const size_t fb = 3 * (size_t)b->cs * b->esz;
   size_t padded = 0;
   for (int i = 0; i < count; ++i) padded += history_bytes(cfgs[i], true);
-  pad = pad && history_fits_padded(padded);
+  const bool pad = !tight && history_fits_padded(padded);
   for (int i = 0; i < count; ++i) {
     ddfd_config c = cfgs[i];
     c.stream = cfgs[0].stream;
@@ -451,8 +452,9 @@ int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool 
     ms.kz = b->kz;
     ms.kz_lean = b->kz_lean;
     ms.tile = b->tile;
+    ms.pad = pad;
     ddfd_problem *p = nullptr;
-    const int st = create_impl(&c, &ms, &p, pad);
+    const int st = create_impl(&c, &ms, &p, tight);
     if (st) return bail(st, "member " + std::to_string(i) + ": " + thread_error());
     b->m.push_back(p);
   }
@@ -468,9 +470,8 @@ int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool 
 extern "C" {
 
 int ddfd_create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out) {
-  int st = create_batch(cfgs, count, out, true);
-  if (st == DDFD_E_OOM && std::any_of(cfgs, cfgs + count, may_pad)) st = create_batch(cfgs, count, out, false);
-  return st;
+  const int st = create_batch(cfgs, count, out, false);
+  return st == DDFD_E_OOM ? create_batch(cfgs, count, out, true) : st;
 }
 
 void ddfd_destroy_batch(ddfd_batch *b) {

@@ -171,7 +171,8 @@ __device__ __forceinline__ void kuhn_rows(const KuhnRowParams<T> &P) {
   }
 }
 
-template <typename T, bool ADJ>
+// RB: rows that a block holds at most, EBE_RB or EBE_RB_TIGHT (summed EBE_RB at a time).
+template <typename T, bool ADJ, int RB>
 __global__ void __launch_bounds__(EBE_THREADS, EBE_CTAS) k_ebe(const __grid_constant__ EbeParams<T> P) {
   extern __shared__ __align__(128) unsigned char sm[];
   __shared__ int s_ok;
@@ -255,28 +256,30 @@ __global__ void __launch_bounds__(EBE_THREADS, EBE_CTAS) k_ebe(const __grid_cons
         st_grad(const_cast<T *>(sG) + 12 * t, o);
       }
       __syncthreads();
-      const int lr = tid / EBE_TPR, j = tid % EBE_TPR;
-      T y[3] = {T(0), T(0), T(0)};
-      if (lr < B.nrows) {
-        for (int e = j; e < B.maxinc; e += EBE_TPR) {
-          const uint16_t code = sI[e * EBE_RB + lr];
-          if (code == EBE_PAD) break;
-          const T *o = sG + 12 * (code >> 2) + 3 * (code & 3);
-          y[0] += o[0];
-          y[1] += o[1];
-          y[2] += o[2];
+      const int j = tid % EBE_TPR;
+      for (int lr = tid / EBE_TPR, r0 = 0; r0 < (RB > EBE_RB ? B.nrows : 1); lr += EBE_RB, r0 += EBE_RB) {
+        T y[3] = {T(0), T(0), T(0)};
+        if (lr < B.nrows) {
+          for (int e = j; e < B.maxinc; e += EBE_TPR) {
+            const uint16_t code = sI[e * RB + lr];
+            if (code == EBE_PAD) break;
+            const T *o = sG + 12 * (code >> 2) + 3 * (code & 3);
+            y[0] += o[0];
+            y[1] += o[1];
+            y[2] += o[2];
+          }
         }
-      }
 #pragma unroll
-      for (int m = 1; m < EBE_TPR; m <<= 1) {
+        for (int m = 1; m < EBE_TPR; m <<= 1) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], m);
-      }
-      if (j == 0 && lr < B.nrows) {
-        const int r = P.blk_rows[B.row0 + lr];
-        const T sc = (T)P.scale[r];  // h^2 / m_a
+          for (int c = 0; c < 3; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], m);
+        }
+        if (j == 0 && lr < B.nrows) {
+          const int r = P.blk_rows[B.row0 + lr];
+          const T sc = (T)P.scale[r];  // h^2 / m_a
 #pragma unroll
-        for (int c = 0; c < 3; ++c) P.out_r[c * (long long)P.n_rows + r] = sc * y[c];
+          for (int c = 0; c < 3; ++c) P.out_r[c * (long long)P.n_rows + r] = sc * y[c];
+        }
       }
       // the next block's copy writes into the other stage; this stage's
       // gradients were overwritten, and its next copy comes after the
@@ -304,59 +307,61 @@ __global__ void __launch_bounds__(EBE_THREADS, EBE_CTAS) k_ebe(const __grid_cons
     __syncthreads();
     // rows: thread j of a row sums its incidences j, j + EBE_TPR, ... (in T:
     // at most a few terms each, as the stencil rows do)
-    const int lr = tid / EBE_TPR, j = tid % EBE_TPR;
-    T y[3] = {T(0), T(0), T(0)}, q[3] = {T(0), T(0), T(0)};
-    if (lr < B.nrows) {
-      for (int e = j; e < B.maxinc; e += EBE_TPR) {
-        const uint16_t code = sI[e * EBE_RB + lr];
-        if (code == EBE_PAD) break;
-        const int t = code >> 2, a = code & 3;
-        T g[12];
-        ld_grad(sG + 12 * t, g);
-        const uint2 nd = sT[t];
-        const int ids[4] = {(int)(nd.x & 0xFFFF), (int)(nd.x >> 16), (int)(nd.y & 0xFFFF), (int)(nd.y >> 16)};
-        // g_a by selection (a dynamic index would put g in local memory)
-        T ga0 = g[0], ga1 = g[1], ga2 = g[2];
+    const int j = tid % EBE_TPR;
+    for (int lr = tid / EBE_TPR, r0 = 0; r0 < (RB > EBE_RB ? B.nrows : 1); lr += EBE_RB, r0 += EBE_RB) {
+      T y[3] = {T(0), T(0), T(0)}, q[3] = {T(0), T(0), T(0)};
+      if (lr < B.nrows) {
+        for (int e = j; e < B.maxinc; e += EBE_TPR) {
+          const uint16_t code = sI[e * RB + lr];
+          if (code == EBE_PAD) break;
+          const int t = code >> 2, a = code & 3;
+          T g[12];
+          ld_grad(sG + 12 * t, g);
+          const uint2 nd = sT[t];
+          const int ids[4] = {(int)(nd.x & 0xFFFF), (int)(nd.x >> 16), (int)(nd.y & 0xFFFF), (int)(nd.y >> 16)};
+          // g_a by selection (a dynamic index would put g in local memory)
+          T ga0 = g[0], ga1 = g[1], ga2 = g[2];
 #pragma unroll
-        for (int b = 1; b < 4; ++b)
-          if (a == b) ga0 = g[3 * b + 0], ga1 = g[3 * b + 1], ga2 = g[3 * b + 2];
-        T lap0 = T(0), lap1 = T(0), lap2 = T(0);
+          for (int b = 1; b < 4; ++b)
+            if (a == b) ga0 = g[3 * b + 0], ga1 = g[3 * b + 1], ga2 = g[3 * b + 2];
+          T lap0 = T(0), lap1 = T(0), lap2 = T(0);
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          T v[4];
-          ld_node(sN + 4 * ids[b], v);
-          const T w = ga0 * g[3 * b + 0] + ga1 * g[3 * b + 1] + ga2 * g[3 * b + 2];
-          lap0 += w * v[0];
-          lap1 += w * v[1];
-          lap2 += w * v[2];
+          for (int b = 0; b < 4; ++b) {
+            T v[4];
+            ld_node(sN + 4 * ids[b], v);
+            const T w = ga0 * g[3 * b + 0] + ga1 * g[3 * b + 1] + ga2 * g[3 * b + 2];
+            lap0 += w * v[0];
+            lap1 += w * v[1];
+            lap2 += w * v[2];
+          }
+          const T div = sD[t];
+          y[0] += lap0;
+          y[1] += lap1;
+          y[2] += lap2;
+          q[0] += ga0 * div;
+          q[1] += ga1 * div;
+          q[2] += ga2 * div;
         }
-        const T div = sD[t];
-        y[0] += lap0;
-        y[1] += lap1;
-        y[2] += lap2;
-        q[0] += ga0 * div;
-        q[1] += ga1 * div;
-        q[2] += ga2 * div;
       }
-    }
-    // the row's partial sums, merged by a butterfly (a + b == b + a, so all
-    // lanes of the row hold the same bits; the order is fixed: reproducible)
+      // the row's partial sums, merged by a butterfly (a + b == b + a, so all
+      // lanes of the row hold the same bits; the order is fixed: reproducible)
 #pragma unroll
-    for (int m = 1; m < EBE_TPR; m <<= 1) {
+      for (int m = 1; m < EBE_TPR; m <<= 1) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        y[c] += __shfl_xor_sync(0xffffffffu, y[c], m);
-        q[c] += __shfl_xor_sync(0xffffffffu, q[c], m);
+        for (int c = 0; c < 3; ++c) {
+          y[c] += __shfl_xor_sync(0xffffffffu, y[c], m);
+          q[c] += __shfl_xor_sync(0xffffffffu, q[c], m);
+        }
       }
-    }
-    if (j == 0 && lr < B.nrows) {
-      const int r = P.blk_rows[B.row0 + lr];
-      const T sc = (T)P.scale[r];  // h^2 / m_a
-      const T sa = ADJ ? node_s(P, P.row_node[r]) : T(1);
+      if (j == 0 && lr < B.nrows) {
+        const int r = P.blk_rows[B.row0 + lr];
+        const T sc = (T)P.scale[r];  // h^2 / m_a
+        const T sa = ADJ ? node_s(P, P.row_node[r]) : T(1);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        P.out_r[c * (long long)P.n_rows + r] = sc * (y[c] + sa * q[c]);
-        if (ADJ) P.out_q[c * (long long)P.n_rows + r] = sc * q[c];
+        for (int c = 0; c < 3; ++c) {
+          P.out_r[c * (long long)P.n_rows + r] = sc * (y[c] + sa * q[c]);
+          if (ADJ) P.out_q[c * (long long)P.n_rows + r] = sc * q[c];
+        }
       }
     }
     st ^= 1;
@@ -373,21 +378,27 @@ void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s, bool chained) {
   if (want <= 0) return;
   const int grid = std::min(want, g_ebe_ctas > 0 ? g_ebe_ctas : 1);
   const size_t smem = 128 + 2 * (size_t)P.stage_bytes;
-  launch_chained(adj ? k_ebe<T, true> : k_ebe<T, false>, dim3((unsigned)grid), EBE_THREADS, smem, s, chained, P);
+  const auto kernel = P.rb > EBE_RB ? (adj ? k_ebe<T, true, EBE_RB_TIGHT> : k_ebe<T, false, EBE_RB_TIGHT>)
+                                    : (adj ? k_ebe<T, true, EBE_RB> : k_ebe<T, false, EBE_RB>);
+  launch_chained(kernel, dim3((unsigned)grid), EBE_THREADS, smem, s, chained, P);
 }
 
 template void launch_ebe<float>(const EbeParams<float> &, bool, cudaStream_t, bool);
 template void launch_ebe<double>(const EbeParams<double> &, bool, cudaStream_t, bool);
+
+template <typename T, int RB>
+static cudaError_t set_ebe_smem(int lim) {
+  const cudaError_t e = cudaFuncSetAttribute(k_ebe<T, false, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k_ebe<T, true, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+}
 
 cudaError_t prepare_ebe_kernels() {
   const int lim = 128 + 2 * EBE_SMEM_BUDGET;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
-      (e = cudaFuncSetAttribute(k_ebe<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
-      (e = cudaFuncSetAttribute(k_ebe<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
-      (e = cudaFuncSetAttribute(k_ebe<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) ||
-      (e = cudaFuncSetAttribute(k_ebe<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)))
+      (e = set_ebe_smem<float, EBE_RB>(lim)) || (e = set_ebe_smem<float, EBE_RB_TIGHT>(lim)) ||
+      (e = set_ebe_smem<double, EBE_RB>(lim)) || (e = set_ebe_smem<double, EBE_RB_TIGHT>(lim)))
     return e;
   g_ebe_ctas = sms > 0 ? EBE_CTAS * sms : 1;
   return cudaSuccess;

@@ -16,16 +16,16 @@ namespace {
 long long align16(long long b) { return (b + 15) & ~15LL; }
 
 // Blob bytes of a block: gradients, local node ids, incidences.
-long long blob_bytes(long long nt, long long maxinc, int esz) {
-  return align16(nt * (12LL * esz + 8) + maxinc * EBE_RB * 2LL);
+long long blob_bytes(long long nt, long long maxinc, int esz, int rb) {
+  return align16(nt * (12LL * esz + 8) + maxinc * rb * 2LL);
 }
 
 }  // namespace
 
-long long ebe_block_smem(long long nt, long long nn, long long maxinc, int esz) {
+long long ebe_block_smem(long long nt, long long nn, long long maxinc, int esz, int rb) {
   nt += nt & 1;
   // blob, node values [nn][4] (field components and s), per-tet divergence
-  return blob_bytes(nt, maxinc, esz) + align16(nn * 4LL * esz) + align16(nt * (long long)esz);
+  return blob_bytes(nt, maxinc, esz, rb) + align16(nn * 4LL * esz) + align16(nt * (long long)esz);
 }
 
 void kuhn_stencil_rows(long long n_grid_rows, int n, const int *rptr, const int *itet, const int *tet_ids,
@@ -67,7 +67,7 @@ void kuhn_stencil_rows(long long n_grid_rows, int n, const int *rptr, const int 
 
 bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const double *tgrad, const int *rptr,
                      const int *itet, const int *iloc, const double *rpos, int esz, EbePack *out, std::string *err,
-                     const unsigned char *use, int max_rows, int budget) {
+                     const unsigned char *use, int max_rows, int budget, int rb) {
   out->blocks.clear();
   out->blob.clear();
   out->nodes.clear();
@@ -106,7 +106,7 @@ bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const d
     const long long nt = (long long)bt.size() + (bt.size() & 1);
     EbeBlock B;
     B.blob = (long long)out->blob.size();
-    B.bytes = (int)blob_bytes(nt, maxinc, esz);
+    B.bytes = (int)blob_bytes(nt, maxinc, esz, rb);
     B.nt = (int)nt;
     B.nn = (int)bn.size();
     B.maxinc = maxinc;
@@ -131,15 +131,15 @@ bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const d
       for (int q = 0; q < 4; ++q) np[4 * i + q] = (uint16_t)locN[tnc[4 * t + q]];
     }
     // the padding tet (zero gradients) points at node 0
-    std::fill(ip, ip + (size_t)maxinc * EBE_RB, EBE_PAD);
+    std::fill(ip, ip + (size_t)maxinc * rb, EBE_PAD);
     for (size_t lr = 0; lr < br.size(); ++lr) {
       const long long r = br[lr];
       for (int e = rptr[r]; e < rptr[r + 1]; ++e)
-        ip[(size_t)(e - rptr[r]) * EBE_RB + lr] = (uint16_t)((locT[itet[e]] << 2) | iloc[e]);
+        ip[(size_t)(e - rptr[r]) * rb + lr] = (uint16_t)((locT[itet[e]] << 2) | iloc[e]);
     }
     for (int c : bn) out->nodes.push_back(uniq[c]);
     for (long long r : br) out->rows.push_back((int)r);
-    out->smem = std::max(out->smem, (int)ebe_block_smem(nt, B.nn, maxinc, esz));
+    out->smem = std::max(out->smem, (int)ebe_block_smem(nt, B.nn, maxinc, esz, rb));
     out->blocks.push_back(B);
     bt.clear();
     bn.clear();
@@ -167,7 +167,7 @@ bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const d
         }
       }
       const long long nt = (long long)(bt.size() + newT.size());
-      const long long bytes = ebe_block_smem(nt, (long long)(bn.size() + newN.size()), std::max(maxinc, deg), esz);
+      const long long bytes = ebe_block_smem(nt, (long long)(bn.size() + newN.size()), std::max(maxinc, deg), esz, rb);
       const bool fits = (long long)br.size() < max_rows && bytes <= budget && nt < (1 << 14);
       if (fits) break;
       if (br.empty()) {

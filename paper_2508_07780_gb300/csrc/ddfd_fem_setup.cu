@@ -66,10 +66,14 @@ int upload_ebe(ddfd_problem *p, long long rows, long long ntet, const std::vecto
   std::string m;
   // (a row with more elements than half an SM's shared memory takes: blocks of the larger budget)
   bool packed = false;
-  for (int budget : {EBE_SMEM_SHARED, EBE_SMEM_BUDGET})
+  p->ebe_rb = p->tight ? EBE_RB_TIGHT : EBE_RB;
+  for (int budget : {EBE_SMEM_SHARED, EBE_SMEM_BUDGET}) {
+    if (p->tight && budget != EBE_SMEM_BUDGET) continue;
     if ((packed = pack_ebe_blocks(rows, ntet, tnode.data(), tgrad.data(), rptr.data(), itet.data(), iloc.data(),
-                                  rpos.data(), (int)p->esz, &pk, &m, stencil ? use.data() : nullptr, max_rows, budget)))
+                                  rpos.data(), (int)p->esz, &pk, &m, stencil ? use.data() : nullptr,
+                                  p->tight ? EBE_RB_TIGHT : max_rows, budget, p->ebe_rb)))
       break;
+  }
   if (!packed) return fail(p, DDFD_E_ARG, m);
   if (!klist.empty()) {
     int st;

@@ -82,7 +82,7 @@ struct ddfd_problem {
   int *ebe_row_node = nullptr, *ebe_blk_nodes = nullptr, *ebe_blk_rows = nullptr;
   ddfd::EbeBlock *ebe_blocks = nullptr;
   unsigned char *ebe_blob = nullptr;
-  int ebe_nblocks = 0, ebe_smem = 0;
+  int ebe_nblocks = 0, ebe_smem = 0, ebe_rb = ddfd::EBE_RB;
   // algorithmic bytes of one step's element-apply launches (forward, adjoint):
   // each gathered tet's node ids and gradients, each of its nodes' values once,
   // each row's outputs; stencil rows their own node values and outputs
@@ -118,6 +118,7 @@ struct ddfd_problem {
   int state = ddfd::host::ST_READY;
   int64_t generation = 0;     // +1 whenever the coefficients or the forward state change
   int64_t launches = 0, fwd_steps = 0;
+  bool tight = false;         // the form that takes the least memory (create_impl)
   ddfd::Tile64 tile;          // FP64 tile shape
   int kz = 16;                // z depth of the step kernel's full items (and of the FP64 kernel's)
   int kz_lean = 16;           // z depth of the FP32 step kernel's lean items
@@ -186,6 +187,7 @@ struct MemberSlot {
   int slot;
   int kz, kz_lean;  // the batch's tile depths
   Tile64 tile;
+  bool pad;         // pad the history's rows where the member may (may_pad)
 };
 
 // Message of the last failing handle-less call in this thread.
@@ -228,6 +230,8 @@ int build_source_table(ddfd_problem *p);
 // Default z depth of the step kernels' items (tile_kz = 0, tile_kz_lean = 0)
 // for `count` problems of n^3 nodes.
 int default_kz(int n, int fp32, int count, Tile64 tile);
+// ... and that of tight handles.
+int tight_kz(int n);
 
 // Dispatch order of one step launch over the problems `ps` (stacked in that
 // order), in z slabs (one problem's z range over a set of its tile columns,
@@ -264,7 +268,11 @@ int validate(const ddfd_config *c, std::string *m);
 int grad_mode(int k, int k_first);
 
 // Single-problem operations (ddfd_api.cu).
-int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out, bool pad);
+// tight: the form of a handle that takes the least memory -- unpadded history rows,
+// FP64 tiles of 32 x 8 nodes and deep items (fewer of them in the dispatch order),
+// gather blocks of EBE_RB_TIGHT rows -- for what does not fit the device or its
+// mem_budget otherwise.  Slower, the same results to the bit.
+int create_impl(const ddfd_config *cfg, const MemberSlot *ext, ddfd_problem **out, bool tight);
 void destroy_problem(ddfd_problem *p);
 void drop_graphs(ddfd_problem *p);
 int sync_check(ddfd_problem *p);
@@ -404,6 +412,7 @@ void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, 
   E.blk_nodes = p->ebe_blk_nodes;
   E.blk_rows = p->ebe_blk_rows;
   E.stage_bytes = p->ebe_smem;
+  E.rb = p->ebe_rb;
   E.err = err ? err : p->errflag;
   E.spin_limit = p->test_spin ? p->test_spin : 1u << 22;
   E.test_skip_copy = p->test_fault;

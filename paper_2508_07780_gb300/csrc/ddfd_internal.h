@@ -172,7 +172,9 @@ int launch_adjoint_step(const StepLaunch<T, NB> &L, cudaStream_t s);
 // nodes), every tet incident to them and every node of those tets; one CTA
 // copies the block's tets into shared memory, gathers its nodes' values, and
 // then sums each row over its incident tets from shared memory only.
-constexpr int EBE_RB = 64;                   // rows per block
+constexpr int EBE_RB = 64;                   // rows per block, and rows summed at a time
+constexpr int EBE_RB_TIGHT = 128;            // rows per block of a handle short of memory: fewer blocks share fewer
+                                             // tets twice (41^3 with a 21^3 cube: 14.1 MB against 16.4)
 constexpr int EBE_TPR = 8;                   // threads per row
 constexpr int EBE_THREADS = EBE_TPR * EBE_RB;
 constexpr int EBE_CTAS = 2;                  // thread blocks per SM: one sums while the other waits (81^3 with
@@ -189,7 +191,8 @@ constexpr uint16_t EBE_PAD = 0xFFFF;         // unused incidence slot
 // its nt tets (nt even; a padding tet has zero gradients), sqrt|K| times the
 // P1 gradients [nt][4][3] (element type T), the tets' local node ids
 // [nt][4] (uint16), and the rows' incidences [maxinc][EBE_RB] (uint16:
-// local tet << 2 | the row's vertex in it, EBE_PAD where a row has fewer).
+// local tet << 2 | the row's vertex in it, EBE_PAD where a row has fewer;
+// EBE_RB_TIGHT rows in tight blocks).
 struct EbeBlock {
   long long blob;  // byte offset of the blob
   int bytes;       // blob size
@@ -213,10 +216,11 @@ struct EbePack {
 };
 bool pack_ebe_blocks(long long n_rows, long long ntet, const int *tnode, const double *tgrad, const int *rptr,
                      const int *itet, const int *iloc, const double *rpos, int esz, EbePack *out, std::string *err,
-                     const unsigned char *use = nullptr, int max_rows = EBE_RB, int budget = EBE_SMEM_BUDGET);
+                     const unsigned char *use = nullptr, int max_rows = EBE_RB, int budget = EBE_SMEM_BUDGET,
+                     int rb = EBE_RB);
 // use (may be NULL: every row): rows with use[r] = 0 are left out of the blocks;
-// max_rows, budget: rows (<= EBE_RB) and bytes of shared memory per block at
-// most.
+// max_rows, budget: rows (<= rb) and bytes of shared memory per block at
+// most; rb: the rows that a block's incidence table has room for.
 
 // Marks the grid rows (the first n_grid_rows rows) whose incident tets are
 // exactly the 24 tets of the uniform Kuhn split around the node: 24 incident
@@ -242,7 +246,7 @@ struct KuhnRowParams {
   T B[8][9];                // (D^T D)_{i,i+o} / h, offsets 0, (1,0,0) (0,1,0) (0,0,1) (1,1,0) (1,0,1) (0,1,1) (1,1,1)
 };
 // Shared-memory bytes of a block with nt tets, nn nodes, maxinc incidences.
-long long ebe_block_smem(long long nt, long long nn, long long maxinc, int esz);
+long long ebe_block_smem(long long nt, long long nn, long long maxinc, int esz, int rb = EBE_RB);
 
 template <typename T>
 struct EbeParams {
@@ -254,6 +258,7 @@ struct EbeParams {
   const unsigned char *blob;
   const int *blk_nodes;     // padded node offsets of the blocks' nodes
   const int *blk_rows;      // row indices of the blocks' rows
+  int rb;                   // rows that the blocks' incidence tables have room for
   int stage_bytes;          // shared memory of one pipeline stage (>= every block's)
   int *err;                 // bit 8: a bounded wait for a block's copy gave up
   uint32_t spin_limit;      // polls per bounded wait
