@@ -135,7 +135,12 @@ template <typename T, bool ADJ>
 __device__ __forceinline__ void kuhn_rows(const KuhnRowParams<T> &P) {
   const long long sx = 1, sy = P.px, sz = (long long)P.px * P.n;
   const long long off[7] = {sx, sy, sz, sx + sy, sx + sz, sy + sz, sx + sy + sz};
-  for (int q = blockIdx.x * EBE_THREADS + threadIdx.x; q < P.n_list; q += gridDim.x * EBE_THREADS) {
+  // a warp takes 32 rows in a row, neighbouring warps' rows go to neighbouring thread
+  // blocks: in FP64 the rows are bound by the SMs' FP64 units and have to spread over all
+  // of them (61^3 with a refined 31^3 cube, FP64: 106 / 90 -> 71 / 72 us a step; FP32 81^3,
+  // 41^3 cube: 19.4 / 21.0 -> 18.2 / 19.7)
+  const int warp = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
+  for (int q = 32 * warp + (int)(threadIdx.x & 31); q < P.n_list; q += (int)gridDim.x * EBE_THREADS) {
     const int r = P.list[q];
     const long long o = P.row_node[r];
     T lap[3], g[3] = {T(0), T(0), T(0)};
@@ -374,7 +379,7 @@ static int g_ebe_ctas = 0;  // EBE_CTAS per SM
 
 template <typename T>
 void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s, bool chained) {
-  const int want = std::max(P.n_blocks, (P.kuhn.n_list + EBE_THREADS - 1) / EBE_THREADS);
+  const int want = std::max(P.n_blocks, (P.kuhn.n_list + 31) / 32);
   if (want <= 0) return;
   const int grid = std::min(want, g_ebe_ctas > 0 ? g_ebe_ctas : 1);
   const size_t smem = 128 + 2 * (size_t)P.stage_bytes;
