@@ -126,7 +126,8 @@ bool history_fits_padded(size_t padded) {
   return padded + total / 16 <= fre;
 }
 
-// At most a 32nd of the memory that is left, and none under a memory budget.
+// At most a 32nd of the memory that is left, and none under a memory budget; else FP32
+// handles keep the flux of SRC_ROWS steps, if that fits.
 int build_source_table(ddfd_problem *p) {
   p->src_off.assign(p->n_src, 0);
   long long steps = 0;
@@ -136,9 +137,11 @@ int build_source_table(ddfd_problem *p) {
   }
   const size_t row = (size_t)p->n * p->px * (p->fp32 ? 3 : 1);
   size_t fre = 0, total = 0;
-  if (steps == 0 || p->cfg.mem_budget > 0) return DDFD_OK;
+  if (steps == 0) return DDFD_OK;
   CK(cudaMemGetInfo(&fre, &total));
-  if ((size_t)steps * row * p->esz > fre / 32 || dalloc(p, (size_t)steps * row * p->esz, &p->src_tab)) {
+  if (p->cfg.mem_budget > 0 || (size_t)steps * row * p->esz > fre / 32 ||
+      dalloc(p, (size_t)steps * row * p->esz, &p->src_tab)) {
+    if (p->fp32) dalloc(p, SRC_ROWS * row * p->esz, (void **)&p->src_rows);
     p->err.clear();
     return DDFD_OK;
   }
@@ -549,7 +552,7 @@ int enqueue_adjoint(ddfd_problem *p, cudaStream_t sm, int64_t *nk) {
         bool chained = false;
         for (int st = n0; st < n1; ++st) {
           // (the trace is written again with the same values)
-          set_forward_step(F, p, s, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs);
+          set_forward_step(F, p, s, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs, n0);
           enqueue_ebe<T>(p, p->E[fc], false, sm, nk, nullptr, nullptr, chained);
           chained = chained || p->ebe_rows > 0;
           *nk += launch_forward_step(single_launch(F, p->mE_halo[fc], p->mE_ctr[fo], p, chained), sm);

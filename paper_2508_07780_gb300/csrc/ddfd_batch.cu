@@ -151,7 +151,7 @@ int enqueue_batch_adjoint(ddfd_batch *b, cudaStream_t sm, int64_t *nk) {
         launch_groups<T>(
             b, false, ck, b->maps.E_halo[fc], b->maps.E_ctr[fo],
             [&](StepParams<T> &P, ddfd_problem *p) {
-              set_forward_step(P, p, 0, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs);
+              set_forward_step(P, p, 0, st, p->E[fc], p->E[fo], (T *)p->hist + (size_t)(st + 1 - n0) * 3 * p->hcs, n0);
             },
             sm, nk, &b->items_ck, st > n0);
         std::swap(fc, fo);

@@ -70,6 +70,7 @@ struct ddfd_problem {
   int hp = 0, hx = 0;
   bool hvec = false;
   long long hcs = 0, hnew = 0;
+  float *src_rows = nullptr;  // FP32 oblique sources without a table: the flux of SRC_ROWS steps
   void *src_tab = nullptr;    // oblique sources (StepParams::src_tab); source s at src_off[s] steps
   std::vector<long long> src_off;
   void *hist_fem = nullptr;   // literal gradient: E on the FEM-updated nodes, every step
@@ -224,7 +225,8 @@ bool may_pad(const ddfd_config &c);
 size_t history_bytes(const ddfd_config &c, bool pad);
 bool history_fits_padded(size_t padded);
 // Tabulates the oblique sources of a handle (after its other allocations; left
-// out, and evaluated in the step kernels, where memory is short).
+// out, and evaluated a few steps at a time or in the step kernels, where memory is
+// short).
 int build_source_table(ddfd_problem *p);
 
 // Default z depth of the step kernels' items (tile_kz = 0, tile_kz_lean = 0)
@@ -347,10 +349,11 @@ void set_source(StepParams<T> &P, const ddfd_problem *p, int s) {
   for (int q = 0; q < 3; ++q) P.pol[q] = p->pol[3 * s + q];
 }
 
-// Per-step scalars of forward step st (E^st -> E^{st+1}) of source s.
+// Per-step scalars of forward step st (E^st -> E^{st+1}) of source s, in a sequence of
+// steps that begins with step `first`.
 template <typename T>
 void set_forward_step(StepParams<T> &P, const ddfd_problem *p, int s, int st, const void *cur, void *old,
-                      T *hist_w) {
+                      T *hist_w, int first = 0) {
   P.cur = (const T *)cur;
   P.old = (T *)old;
   P.abs_now = faces_at(p, s, st);
@@ -362,6 +365,14 @@ void set_forward_step(StepParams<T> &P, const ddfd_problem *p, int s, int st, co
   // (source s of the handle: set_source has set P.oblique)
   const size_t row = (size_t)p->n * p->px * (p->fp32 ? 3 : 1);
   P.src_tab = p->src_tab && P.oblique && P.src_on ? (const T *)p->src_tab + (size_t)(p->src_off[s] + st) * row : nullptr;
+  P.src_fill = nullptr;
+  if (p->src_rows && P.oblique && P.src_on) {
+    const int j = (st - first) % SRC_ROWS;
+    P.src_tab = (const T *)(p->src_rows + j * row);
+    if (j == 0) P.src_fill = p->src_rows;
+    P.st = st;
+    P.tau = p->tau;
+  }
 }
 
 // Per-step scalars of adjoint step k (mu^k -> mu^{k-1}) of source s.

@@ -44,6 +44,10 @@ struct Tile64 {
 // FP64 tile of `count` problems of n^3 nodes stepped together.
 Tile64 tile64(int n, int count);
 
+// FP32 oblique sources without a table of every step: steps whose flux is evaluated
+// together.
+constexpr int SRC_ROWS = 8;
+
 // FP32 gradient accumulation: the adjoint steps of each block of GRAD_BLOCK
 // consecutive time steps are summed in FP32 (per free node) and the block sum
 // is added to the FP64 accumulators; gmode tells a launch where it sits.
@@ -96,10 +100,12 @@ struct StepParams {
   const T *hist_r;       // adjoint: hist[k]
   long long hcs;
   int hx, hp, hvec;
-  // oblique source of this step, tabulated at creation (null: evaluated in
-  // the kernel): FP32 the three components' flux terms [3][n][px], FP64 the
+  // oblique source of this step, tabulated (null: evaluated in the kernel): FP32 the three components' flux terms [3][n][px], FP64 the
   // pulse times src_scale [n][px]
   const T *src_tab;
+  float *src_fill;       // FP32: the table of SRC_ROWS steps that this step begins, to be filled before it (else null)
+  int st;                // ... its step and the time step
+  double tau;
   double *gacc_e;        // adjoint: gradient accumulators (FP64)
   double *gacc_s;
   // element-by-element FEM rows (fem_kind = DDFD_FEM_EBE): when ebe_r is set,

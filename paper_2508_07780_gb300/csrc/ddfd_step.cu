@@ -855,8 +855,37 @@ template <bool ADJ, int NB>
 static int launch_step(const StepLaunch<double, NB> &L, cudaStream_t s) {
   return launch_step64<ADJ, NB>(L, s);
 }
+// The oblique flux of SRC_ROWS steps of the problems that ask for it, one node and step a
+// thread.  In the step kernel the 512 FP64 sines and exponentials of a top tile hold one
+// SM up for 12 us; here they spread over all SMs, and what a thread waits for, 8 us of
+// FP64 latency, is paid once in SRC_ROWS steps (us a forward step, 41^3 / 81^3 / 121^3:
+// 13.7 / 19.9 / 34.9 -> 6.5 / 12.0 / 25.2; one step at a time 6.2 / 17.5 / 26.1; a table
+// of every step 5.0 / 8.2 / 19.9).
+template <int NB>
+__global__ void __launch_bounds__(128) k_source_rows(const __grid_constant__ StepLaunch<float, NB> L) {
+  pdl_launch_dependents();
+  const StepParams<float> &P = L.p[NB == 1 ? 0 : blockIdx.y];
+  const int n = P.n, q = (int)(blockIdx.x * 128 + threadIdx.x), j = q / (n * n), d = q - j * n * n, y = d / n, x = d - n * y;
+  const bool mine = j < SRC_ROWS && P.src_fill;
+  double v = 0.0;
+  if (mine) v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width, __dmul_rn((double)(P.st + j), P.tau) - P.delay[d]);
+  pdl_wait();  // (the step before reads the table)
+  if (mine)
+    for (int c = 0; c < 3; ++c) P.src_fill[x + P.px * (y + (long long)n * (3 * j + c))] = (float)(P.pol[c] * v);
+}
+
 template <bool ADJ, int NB>
 static int launch_step(const StepLaunch<float, NB> &L, cudaStream_t s) {
+  bool rows = false;
+  for (int q = 0; q < L.nprob && !ADJ; ++q) rows |= L.p[q].src_fill != nullptr;
+  if (rows) {
+    const int total = L.p[0].n * L.p[0].n * SRC_ROWS;
+    launch_chained(k_source_rows<NB>, dim3((unsigned)((total + 127) / 128), (unsigned)L.nprob), 128, 0, s, L.chained != 0, L);
+    StepLaunch<float, NB> M = L;
+    for (int q = 0; q < L.nprob; ++q) M.p[q].src_fill = nullptr;
+    M.chained = 1;
+    return 1 + launch_step<ADJ, NB>(M, s);
+  }
   bool gen = false;
   for (int q = 0; q < L.nprob; ++q) {
     const StepParams<float> &P = L.p[q];
@@ -895,7 +924,8 @@ __global__ void k_source_table(const __grid_constant__ StepParams<T> P, int step
   const long long per = (long long)P.n * P.n, total = per * steps;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total; q += (long long)gridDim.x * blockDim.x) {
     const int st = (int)(q / per), d = (int)(q - per * st), y = d / P.n, x = d - P.n * y;
-    const double v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width, st * tau - P.delay[d]);
+    // (the product rounded as the step kernels' t_n is: the same flux to the bit)
+    const double v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width, __dmul_rn((double)st, tau) - P.delay[d]);
     T *o = out + (long long)st * NC * P.n * P.px + x + P.px * y;
     if (NC == 1)
       o[0] = (T)v;
