@@ -293,6 +293,13 @@ int ddfd_test_gather_timeout(ddfd_problem *p, int32_t fault, uint32_t spin_limit
 int ddfd_test_step_items(int32_t n, int32_t precision, int32_t nprob, const int32_t *boxes, int32_t kz,
                          int32_t kz_lean, uint32_t *items, int64_t cap, int64_t *n_items, int64_t *n_full);
 
+/* Host-only test hook (no GPU): the same for an FP64 launch, on the tiles that it
+ * runs on: 8 x 8 or 14 x 9 nodes, 32 x 8 beyond 448 nodes an axis.  tile[0], tile[1]
+ * receive the tile's width and height; an item's tile x and y count tiles of that size.
+ * Errors as above. */
+int ddfd_test_step_items64(int32_t n, int32_t nprob, const int32_t *boxes, int32_t kz, int32_t *tile, uint32_t *items,
+                           int64_t cap, int64_t *n_items);
+
 /* Tile autotuner for the step kernels of one handle.  Times `steps` forward
  * and `steps` adjoint steps (CUDA events on the handle's stream, launched as a
  * solve launches them) with the handle's z depth of the full items and with

@@ -39,7 +39,7 @@ ABI_SYMBOLS = (
     "ddfd_batch_member", "ddfd_batch_forward", "ddfd_batch_forward_dev", "ddfd_batch_adjoint",
     "ddfd_batch_adjoint_dev", "ddfd_batch_autotune", "ddfd_batch_get_info",
     "ddfd_cg_params_default", "ddfd_cg_run", "ddfd_test_gather_timeout", "ddfd_time_gather",
-    "ddfd_test_step_items",
+    "ddfd_test_step_items", "ddfd_test_step_items64",
 )
 
 
@@ -161,6 +161,8 @@ def load_library(path: str = LIB_PATH):
     lib.ddfd_batch_autotune.argtypes = [P, c_int32, POINTER(c_int32)]
     lib.ddfd_batch_get_info.argtypes = [P, POINTER(ddfd_batch_info)]
     lib.ddfd_test_gather_timeout.argtypes = [P, c_int32, ctypes.c_uint32]
+    lib.ddfd_test_step_items64.argtypes = [c_int32, c_int32, POINTER(c_int32), c_int32, POINTER(c_int32),
+                                           POINTER(ctypes.c_uint32), c_int64, POINTER(c_int64)]
     lib.ddfd_test_step_items.argtypes = [c_int32, c_int32, c_int32, POINTER(c_int32), c_int32, c_int32,
                                          POINTER(ctypes.c_uint32), c_int64, POINTER(c_int64), POINTER(c_int64)]
     lib.ddfd_time_gather.argtypes = [P, c_int32, P, P, P, P]
@@ -236,6 +238,23 @@ def step_items(n, precision, boxes, kz, kz_lean):
     if st != DDFD_OK:
         raise DDFDError(st, "ddfd_test_step_items rejected its arguments")
     return out, nf.value
+
+
+def step_items64(n, boxes, kz):
+    """ddfd_test_step_items64 (host only): the dispatch items of an FP64 step launch
+    on the tiles that it runs on.  Returns (items as a uint32 array, (tile width, height))."""
+    lib = load_library()
+    bx = np.ascontiguousarray(np.asarray(boxes, dtype=np.int32).reshape(-1))
+    ni, tile = c_int64(), (c_int32 * 2)()
+    args = (int(n), len(boxes), bx.ctypes.data_as(POINTER(c_int32)), int(kz), tile)
+    out = np.zeros(0, dtype=np.uint32)
+    for _ in range(2):  # the count, then the items
+        ptr = out.ctypes.data_as(POINTER(ctypes.c_uint32)) if out.size else None
+        if lib.ddfd_test_step_items64(*args, ptr, out.size, ctypes.byref(ni)) != DDFD_OK:
+            raise DDFDError(DDFD_E_ARG, "ddfd_test_step_items64 rejected its arguments")
+        if not out.size:
+            out = np.zeros(ni.value, dtype=np.uint32)
+    return out, (tile[0], tile[1])
 
 
 def make_config(lib, kw, keep):
