@@ -70,20 +70,24 @@ void dfree(ddfd_problem *p, void *ptr) {
 // FP64: the step is bound by the SMs' FP64 units: 8 x 8 tiles (small grids) go
 // plane by plane, the others by about 1300 items, 12 planes each at most: deeper
 // items save halo planes and the Gauss-law term's extra layer per item, but end
-// less evenly.  us a step (forward / adjoint): 51^3 23.8 / 23.7, 27.9 / 30.5 (1,
-// 2 planes); 65^3 38.5 / 37.0, 32.1 / 31.5 (1, 2); 100^3 106 / 112, 103 / 108
-// (4, 6); 161^3 466 / 518, 458 / 510 (8, 12).
+// less evenly.  us a step (forward / adjoint): 51^3 18.8 / 19.2, 24.8 / 25.1 (1,
+// 2 planes); 65^3 34.6 / 34.5, 29.3 / 30.8, 45.9 / 43.1 (1, 2, 4); 100^3 97.5 / 101,
+// 93.7 / 98.0, 120 / 142 (4, 6, 12); 161^3 463 / 516, 456 / 508 (8, 12).
 // FP32: two to three items per resident thread block (152 SMs x 2), two planes
 // an item at least: an item starts with the latency of its first planes, which
 // deep items spread, and a step ends when the last item does, which shallow
-// ones bring forward.  us a step (forward / adjoint) at 2, 3, 4, 6, 8, 10, 16
-// planes: 41^3 5.0, 6.2, 7.6 (forward); 65^3 7.2, 8.9 (forward); 100^3 -, -,
-// 13.9 / 14.8, 13.0 / 16.5, -, 19.0 / 24.3; 161^3 with a 121^3 cube 52.0 / 58.5
-// (8), 51.3 / 58.0 (10), 52.9 / 59.3 (16).  Batches of 100 planes and more for
+// ones bring forward.  us a step (forward / adjoint) at 2, 3, 4 planes: 41^3
+// 5.0 / 4.7, 5.9 / 5.8, 7.2 / 7.0; 65^3 5.7 / 6.4, 7.4 / 7.1, 8.6 / 8.4; at 3, 4, 6, 8:
+// 100^3 13.4 / 13.3, 13.0 / 13.0, 12.9 / 12.0, 16.2 / 14.9; 161^3 with a 121^3 cube
+// 49.2 / 53.4 (8), 47.9 / 52.4 (12), 49.3 / 53.9 (16), 51.4 / 53.3 (24); 201^3 60.8 / 65.4
+// (12), 58.2 / 63.6 (16).  Batches of 100 planes and more for
 // each of 720 blocks have so many items that their end is even at 24 planes as
-// well, which save halo planes: 16 x 161^3 544 / 578 (16), 530 / 568 (24),
-// 544 / 582 (32).  One large problem gains nothing: 301^3 182 / 193 and 181 / 194
-// (16, 24), 401^3 380 / 386 and 382 / 389.
+// well, which save halo planes (at 16, 24, 32 planes; planes per block in brackets):
+// 16 x 161^3 (197) 545 / 583, 532 / 572, 545 / 587; 9 x 161^3 (111) 316 / 341, 310 / 336,
+// 318 / 345; 8 x 241^3 (343) 865 / 944, 851 / 934, 843 / 928.  Below that they gain up to
+// 1.5 % or lose: 8 x 161^3 (98) 277 / 297, 272 / 293; 16 x 97^3 (45) 139 / 149, 140 / 150;
+// 2 x 161^3 (25) 91 / 101, 90 / 105.  One problem of as many planes gains nothing: 301^3
+// (79) 185 / 196, 183 / 195, 401^3 (188) 425 / 455, 425 / 455, 501^3 (356) 836 / 885, 835 / 885.
 int default_kz(int n, int fp32, int count, Tile64 tile) {
   const long long tx = fp32 ? step_tiles_x(n) : (n + tile.w - 1) / tile.w;
   const long long ty = fp32 ? step_tiles_y(n) : (n + tile.h - 1) / tile.h;
@@ -207,8 +211,8 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
         }
     }
     // chunks of kz planes, the last one the rest: a short item at the end of a
-    // column helps the step to end evenly (201^3: 61 / 67 us a forward / adjoint
-    // step, with even chunks 64 / 67)
+    // column helps the step to end evenly (with even chunks 201^3 took 3 us more a
+    // forward step, the adjoint the same)
     auto cut = [&](int lo, int hi, bool fem) {
       for (int z0 = lo; z0 < hi; z0 += kz) full.push_back({cost(z0, std::min(z0 + kz, hi)), (int)q, z0, std::min(z0 + kz, hi), fem});
     };
@@ -264,7 +268,7 @@ std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &p
     };
     std::stable_sort(out.begin(), out.end(), [&](uint32_t l, uint32_t r) { return dear(l) > dear(r); });
   }
-  *n_full = (int)out.size();
+  if (n_full) *n_full = (int)out.size();
   // lean items: every node's work is the same, so they go by problem and z
   // chunk (chunks of kz_lean from z = 0), all the chunk's columns together,
   // which keeps the planes that neighbouring items share (x, y and z halos)
@@ -303,8 +307,7 @@ int build_items(ddfd_problem *p) {
     p->items_kz = 0;
   }
   if (!items_fit(p->n, p->kz, p->kz_lean)) return DDFD_OK;  // beyond the item packing: grid order
-  int n_full = 0;
-  const std::vector<uint32_t> it = step_item_order({p}, p->kz, p->kz_lean, &n_full);
+  const std::vector<uint32_t> it = step_item_order({p}, p->kz, p->kz_lean);
   int st = dalloc_t(p, it.size(), &p->items);
   if (st) return st;
   CK(cudaMemcpy(p->items, it.data(), it.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));

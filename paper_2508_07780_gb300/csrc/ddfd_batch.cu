@@ -41,8 +41,7 @@ int build_batch_items(ddfd_batch *b) {
     for (size_t g0 = 0; g0 < lt.first->size(); g0 += BATCH_MAX) {
       std::vector<const ddfd_problem *> ps;
       for (size_t g = g0; g < std::min(g0 + BATCH_MAX, lt.first->size()); ++g) ps.push_back(b->m[(*lt.first)[g]]);
-      int n_full = 0;
-      const std::vector<uint32_t> it = step_item_order(ps, b->kz, b->kz_lean, &n_full);
+      const std::vector<uint32_t> it = step_item_order(ps, b->kz, b->kz_lean);
       uint32_t *d = nullptr;
       if (cudaMalloc((void **)&d, it.size() * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();

@@ -247,7 +247,7 @@ int tight_kz(int n);
 // items' work, heaviest first) and each problem's slabs in ascending z, so that
 // tiles sharing halo planes run close together in time.
 std::vector<uint32_t> step_item_order(const std::vector<const ddfd_problem *> &ps, int kz, int kz_lean,
-                                      int *n_full);
+                                      int *n_full = nullptr);
 // (Re)builds p->items for p->kz and p->kz_lean.
 int build_items(ddfd_problem *p);
 // (Re)builds the batch's tables for b->kz.

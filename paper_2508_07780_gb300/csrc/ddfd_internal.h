@@ -33,9 +33,9 @@ bool invert4(const double A[4][4], double X[4][4]);
 // kernels (cudaErrorInvalidValue if they differ).
 cudaError_t check_kuhn_blocks(const KuhnBlocks &kb, cudaStream_t s);
 
-// Step-kernel tiling.  FP32: a CTA of 256 computing threads owns a 32 x 16
-// (x, y) tile of one z chunk, two x-adjacent nodes per thread.  FP64: one node
-// per thread, a tile shape by the grid's size (tile64).
+// Step-kernel tiling.  FP32: a CTA of 128 computing threads owns a 32 x 16
+// (x, y) tile of one item's planes, four x-adjacent nodes per thread.  FP64: one
+// node per thread, a tile shape by the grid's size (tile64).
 constexpr int STEP_TX = 32;
 constexpr int STEP_TY = 16;
 struct Tile64 {

@@ -23,9 +23,9 @@
 // first planes of an item and the last items of a step -- and the instructions of
 // the FEM rows.  us a step, forward / adjoint, against two launches side by side
 // (two nodes a thread, a kernel for the FEM items and one for the others):
-// 201^3 / 101^3 66 / 71 -> 59 / 64, 301^3 / 151^3 190 / 197 -> 182 / 193,
-// 16 x 161^3 (oblique) 597 / 650 -> 530 / 568, 100^3 / 63^3 18 / 19 -> 13.0 / 13.4,
-// 41^3 / 21^3 10.5 / 11.5 -> 5.1 / 5.0.  Tried and dropped: the last warp to
+// 201^3 / 101^3 66 / 71 -> 58 / 64, 301^3 / 151^3 190 / 197 -> 181 / 192,
+// 16 x 161^3 (oblique) 597 / 650 -> 527 / 568, 100^3 / 63^3 18 / 19 -> 13.0 / 13.0,
+// 41^3 / 21^3 10.5 / 11.5 -> 5.0 / 4.7.  Tried and dropped: the last warp to
 // release a slot staging the next plane instead of a producer warp (301^3
 // without a cube 156 -> 180), two nodes a thread (173), carrying the stencil's
 // lower plane in registers (no gain), s = eps - 1 held for all three components
@@ -169,12 +169,6 @@ __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-#define kOne f2(1.f)
-#define kZero f2(0.f)
-#define kM1 f2(-1.f)
-#define kM6 f2(-6.f)
-#define kSixth f2(1.f / 6.f)
-#define kMSixth f2(-1.f / 6.f)
 
 // The four nodes of a thread: l holds nodes 0 and 1, h nodes 2 and 3.
 struct Quad {
@@ -205,7 +199,7 @@ __device__ __forceinline__ void set(Quad &q, int j, float v) {
 __device__ __forceinline__ float2 wacc2(float2 acc, int w, float2 v) {
   if (w == 0) return acc;
   if (w == 1) return add2(acc, v);
-  if (w == -1) return fma2(v, kM1, acc);
+  if (w == -1) return fma2(v, f2(-1.f), acc);
   return fma2(f2((float)w), v, acc);
 }
 
@@ -346,7 +340,7 @@ __device__ __forceinline__ Quad neg_lap(const Quad &cen, float cm, float cp, con
     if (x + 3 == n - 1) s3 = cen.h.x + cen.h.x;
   }
   const Quad sn = {make_float2(s0, s1), make_float2(s2, s3)};
-  return fma4(cen, kM6, add4(add4(add4(add4(sn, yp), ym), ab), below));
+  return fma4(cen, f2(-6.f), add4(add4(add4(add4(sn, yp), ym), ab), below));
 }
 
 // E^{n+1} = E^n + A (E^n - E^{n-1}) + B E^n - C R, with Q = -R already scaled by
@@ -357,10 +351,10 @@ __device__ __forceinline__ Quad neg_lap(const Quad &cen, float cm, float cp, con
 // 8e-6.
 __device__ __forceinline__ Quad update(const Quad &cen, const Quad &od, const Quad &Q, const Quad &A, const Quad &B,
                                        const Quad &C) {
-  return add4(cen, add4(mul4(A, fma4(od, kM1, cen)), fma4(C, Q, mul4(B, cen))));
+  return add4(cen, add4(mul4(A, fma4(od, f2(-1.f), cen)), fma4(C, Q, mul4(B, cen))));
 }
 __device__ __forceinline__ Quad update(const Quad &cen, const Quad &od, const Quad &Q) {  // A = 1, B = 0, C = 1
-  return add4(cen, add4(fma4(od, kM1, cen), Q));
+  return add4(cen, add4(fma4(od, f2(-1.f), cen), Q));
 }
 
 // GEN: the launch may hold problems with element-gather rows, unpadded history
@@ -563,7 +557,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
   if (!full) {
     // finite-difference nodes only
     // side faces: the coefficients of every plane but the first and last
-    Quad SA = {kOne, kOne}, SB = {kZero, kZero}, SC = {kOne, kOne};
+    Quad SA = {f2(1.f), f2(1.f)}, SB = {f2(0.f), f2(0.f)}, SC = {f2(1.f), f2(1.f)};
     if (colbnd) {
       Quad none[3];
       boundary_quad(1, none, SA, SB, SC);
@@ -635,8 +629,8 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
         const float *hr = P.hist_r + hq, *g = P.gpart + 2 * (long long)hq;
         const bool sums = fre && !(P.gmode & GM_FIRST);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) hv[c] = {kZero, kZero};
-        gp[0] = gp[1] = {kZero, kZero};
+        for (int c = 0; c < 3; ++c) hv[c] = {f2(0.f), f2(0.f)};
+        gp[0] = gp[1] = {f2(0.f), f2(0.f)};
         if (!GEN || P.hvec) {
           if (fre) {
 #pragma unroll
@@ -676,7 +670,7 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
       // boundary terms.
       Quad Q[3], O[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) O[c] = {kZero, kZero};
+      for (int c = 0; c < 3; ++c) O[c] = {f2(0.f), f2(0.f)};
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const float *e = E0 + c * RE;
@@ -708,35 +702,35 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
       Quad od[3], nw[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) od[c] = ld4(C0 + c * TXY);
-      Quad A = {kOne, kOne}, B = {kZero, kZero}, C = {kOne, kOne};
-              if (fem) {
-                A = ld4(C0 + S::Q_OFF / 4);
-                C = ld4(C0 + S::Q_OFF / 4 + TXY);
-                if (GEN && P.ebe_r) {
-                  // element-by-element rows computed by k_ebe for this step
-                  const int fm = P.b - P.a - 1;
-                  const long long row = (x - P.a - 1) + (long long)fm * ((y - P.a - 1) + (long long)fm * (k - P.a - 1));
+      Quad A = {f2(1.f), f2(1.f)}, B = {f2(0.f), f2(0.f)}, C = {f2(1.f), f2(1.f)};
+      if (fem) {
+        A = ld4(C0 + S::Q_OFF / 4);
+        C = ld4(C0 + S::Q_OFF / 4 + TXY);
+        if (GEN && P.ebe_r) {
+          // element-by-element rows computed by k_ebe for this step
+          const int fm = P.b - P.a - 1;
+          const long long row = (x - P.a - 1) + (long long)fm * ((y - P.a - 1) + (long long)fm * (k - P.a - 1));
 #pragma unroll
-                  for (int j = 0; j < 4; ++j)
-                    if (x + j > P.a && x + j < P.b) {
+          for (int j = 0; j < 4; ++j)
+            if (x + j > P.a && x + j < P.b) {
 #pragma unroll
-                      for (int c = 0; c < 3; ++c) {
-                        set(Q[c], j, -P.ebe_r[c * P.ebe_rows + row + j]);
-                        if (ADJ) set(O[c], j, P.ebe_q[c * P.ebe_rows + row + j]);
-                      }
-                    }
-                } else if (!ADJ) {
-#pragma unroll
-                  for (int c = 0; c < 3; ++c) Q[c] = fma4(O[c], kMSixth, Q[c]);
-                } else if (gauss) {
-                  const Quad ns0 = mul4(sc, kM1);
-#pragma unroll
-                  for (int c = 0; c < 3; ++c) {
-                    O[c] = mul4(O[c], kSixth);  // kept for the gradient
-                    Q[c] = fma4(ns0, O[c], Q[c]);
-                  }
-                }
+              for (int c = 0; c < 3; ++c) {
+                set(Q[c], j, -P.ebe_r[c * P.ebe_rows + row + j]);
+                if (ADJ) set(O[c], j, P.ebe_q[c * P.ebe_rows + row + j]);
               }
+            }
+        } else if (!ADJ) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) Q[c] = fma4(O[c], f2(-1.f / 6.f), Q[c]);
+        } else if (gauss) {
+          const Quad ns0 = mul4(sc, f2(-1.f));
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            O[c] = mul4(O[c], f2(1.f / 6.f));  // kept for the gradient
+            Q[c] = fma4(ns0, O[c], Q[c]);
+          }
+        }
+      }
 #pragma unroll
       for (int c = 0; c < 3; ++c) Q[c] = mul4(Q[c], R2);
       if (colbnd || kbnd) boundary_quad(k, Q, A, B, C);
@@ -767,12 +761,12 @@ __global__ void __launch_bounds__(QUAD_THREADS, 2) k_step_quad(const __grid_cons
         } else {
           // the nodes' gradient terms in packed FP32 (at a node that is not free
           // they land in the rows' padding, or are not stored)
-          Quad ge = {kZero, kZero}, gs = {kZero, kZero};
+          Quad ge = {f2(0.f), f2(0.f)}, gs = {f2(0.f), f2(0.f)};
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
             const Quad te = fma4(O[c], R2, add4(fma4(cen[c], f2(-2.f), nw[c]), od[c]));
             ge = fma4(hv[c], te, ge);
-            gs = fma4(hv[c], fma4(od[c], kM1, nw[c]), gs);
+            gs = fma4(hv[c], fma4(od[c], f2(-1.f), nw[c]), gs);
           }
           // block sums in FP32, folded into the FP64 accumulators
           const Quad g0 = {make_float2(ge.l.x, gs.l.x), make_float2(ge.l.y, gs.l.y)};

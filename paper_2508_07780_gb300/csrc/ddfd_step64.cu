@@ -24,7 +24,7 @@
 //
 // Measured (us a step, forward and adjoint averaged, against the 15-point
 // stencil on full 32 x 8 warps with 8 or 16 planes an item): 161^3 with a
-// 121^3 cube 840 -> 484 (the FP64 instructions alone would take about 425),
+// 121^3 cube 840 -> 482 (the FP64 instructions alone would take about 425),
 // 41^3 / 21^3 88 -> 14, 13^3 / 9^3 50 -> 8.  Each step is launched as the last
 // one's programmatic dependent (its barriers and descriptors are set up while
 // that one drains).  So a step may start while the step that writes its fields or
@@ -482,11 +482,11 @@ cudaError_t prepare_step64_kernels() {
 }
 
 // 14 x 9 tiles: 126 of 128 lanes, warps of their own for the halo nodes, 3
-// thread blocks per SM.  Small grids take 8 x 8 (41^3 13.8 / 14.0 us a forward /
+// thread blocks per SM.  Small grids take 8 x 8 (41^3 13.5 / 14.3 us a forward /
 // adjoint step against 18.5 / 19.1; 51^3 even): the FEM cube's nodes, three times
 // as dear as the others, then spread over more SMs.  32 x 8, two thread blocks per
-// SM (161^3 with a 121^3 cube 530 / 591 us against 458 / 510; 65^3 85 / 96
-// against 32 / 32), is left for the grids whose 14-node columns the dispatch
+// SM (161^3 with a 121^3 cube 530 / 591 us against 456 / 508; 65^3 85 / 96
+// against 29 / 31), is left for the grids whose 14-node columns the dispatch
 // items cannot count.
 Tile64 tile64(int n, int count) {
   const long long items = (long long)((n + 7) / 8) * ((n + 7) / 8) * n * count;

@@ -31,11 +31,8 @@ __device__ __forceinline__ int face_count(int i, int j, int k, int n, uint32_t a
   return f;
 }
 
-// FP64 (the FP32 kernel stages its two rings itself): stages plane p = kk - (k0 - 1) of the chunk into slot p % RING and arms the
-// slot's "full" barrier with the byte count: the current level (halo box;
-// mirrored ghost planes at kk = -1 and kk = n), the previous level (centre
-// box, computed planes only) and, on tiles touching the FEM cube, s (halo
-// box, planes a..b) and (q1, q2) (centre box, computed planes a..b).
+// FP64 (the FP32 kernel stages its two rings itself): starts the copies of plane p of
+// produce_planes and arms its slot's "full" barrier with their bytes.
 template <class S>
 __device__ __forceinline__ void stage_plane(int p, const CUtensorMap *mcur, const CUtensorMap *mold,
                                             const CUtensorMap *ms, const CUtensorMap *mq, unsigned char *smem,
