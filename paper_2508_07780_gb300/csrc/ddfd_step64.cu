@@ -415,10 +415,16 @@ __global__ void __launch_bounds__(Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, T
 #pragma unroll
         for (int c = 0; c < 3; ++c) t[c] = dv[c] - P.r2 * R[c];
       }
+      const long long fi = (x - P.f0) + (long long)P.nf * ((y - P.f0) + (long long)P.nf * (k - P.f0));
+      double hv[3] = {0.0, 0.0, 0.0}, ae = 0.0, as = 0.0;  // (read ahead of the stores, which they may not be moved across)
+      if (ADJ && fre) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) hv[c] = P.hist_r[c * P.hcs + fi];
+        ae = P.gacc_e[fi], as = P.gacc_s[fi];
+      }
 #pragma unroll
       for (int c = 0; c < 3; ++c) out[c * cs] = cen[c] + t[c];
       if (fre) {
-        const long long fi = (x - P.f0) + (long long)P.nf * ((y - P.f0) + (long long)P.nf * (k - P.f0));
         if (!ADJ) {
           if (P.hist_w)
 #pragma unroll
@@ -428,12 +434,11 @@ __global__ void __launch_bounds__(Stage64<TW, TH>::CONSUMERS + 32, Stage64<TW, T
           double ge = 0.0, gs = 0.0;
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const double hv = P.hist_r[c * P.hcs + fi];
-            ge += hv * ((t[c] - dv[c]) + sx[c]);
-            gs += hv * (t[c] + dv[c]);
+            ge += hv[c] * ((t[c] - dv[c]) + sx[c]);
+            gs += hv[c] * (t[c] + dv[c]);
           }
-          P.gacc_e[fi] += ge;
-          P.gacc_s[fi] += gs;
+          P.gacc_e[fi] = ae + ge;
+          P.gacc_s[fi] = as + gs;
         }
       }
     }
