@@ -130,6 +130,17 @@ bool history_fits_padded(size_t padded) {
   return padded + total / 16 <= fre;
 }
 
+// us a forward step with the flux evaluated before the step, in the step kernel: 81^3
+// 11.6, 21.2; 301^3 193, 199; 401^3 442, 447; 5 x 81^3 34, 45; 16 x 65^3 64, 70;
+// 6 x 161^3 218, 217; 16 x 161^3 546, 528: the FP64 units take 4 us for 161^2 nodes, which
+// the steps of large batches hide.  One of five 81^3 34, 32; one of 16 x 65^3 61, 59; one
+// of two 100^3 28, 31: few nodes' pulses hide in a step of many items.
+bool source_rows_pay(int n, int asking, int count) {
+  const long long nodes = (long long)n * n * std::min(asking, BATCH_MAX);
+  const long long planes = (long long)step_tiles_x(n) * step_tiles_y(n) * n * std::min(count, BATCH_MAX);
+  return nodes <= 150000 && (asking == count || planes < 9 * 720);
+}
+
 // At most a 32nd of the memory that is left, and none under a memory budget; else FP32
 // handles keep the flux of SRC_ROWS steps, if that fits.
 int build_source_table(ddfd_problem *p) {
@@ -145,7 +156,7 @@ int build_source_table(ddfd_problem *p) {
   CK(cudaMemGetInfo(&fre, &total));
   if (p->cfg.mem_budget > 0 || (size_t)steps * row * p->esz > fre / 32 ||
       dalloc(p, (size_t)steps * row * p->esz, &p->src_tab)) {
-    if (p->fp32) dalloc(p, SRC_ROWS * row * p->esz, (void **)&p->src_rows);
+    if (p->fp32 && source_rows_pay(p->n, 1, 1)) dalloc(p, SRC_ROWS * row * p->esz, (void **)&p->src_rows);
     p->err.clear();
     return DDFD_OK;
   }

@@ -460,6 +460,14 @@ int create_batch(const ddfd_config *cfgs, int32_t count, ddfd_batch **out, bool 
   if (build_batch_items(b)) return bail(DDFD_E_OOM, b->err);
   for (ddfd_problem *p : b->m)
     if (const int st = build_source_table(p)) return bail(st, p->err);
+  int asking = 0;
+  for (ddfd_problem *p : b->m) asking += p->src_rows != nullptr;
+  if (asking && !source_rows_pay(b->n, asking, count))
+    for (ddfd_problem *p : b->m)
+      if (p->src_rows) {
+        dfree(p, p->src_rows);
+        p->src_rows = nullptr;
+      }
   *out = b;
   return DDFD_OK;
 }

@@ -224,6 +224,9 @@ void dfree(ddfd_problem *p, void *ptr);
 bool may_pad(const ddfd_config &c);
 size_t history_bytes(const ddfd_config &c, bool pad);
 bool history_fits_padded(size_t padded);
+// Whether `asking` of `count` FP32 problems of n^3 nodes, whose oblique sources have no
+// table, have their flux evaluated before the step (SRC_ROWS steps at a time) or in it.
+bool source_rows_pay(int n, int asking, int count);
 // Tabulates the oblique sources of a handle (after its other allocations; left
 // out, and evaluated a few steps at a time or in the step kernels, where memory is
 // short).
@@ -365,13 +368,11 @@ void set_forward_step(StepParams<T> &P, const ddfd_problem *p, int s, int st, co
   // (source s of the handle: set_source has set P.oblique)
   const size_t row = (size_t)p->n * p->px * (p->fp32 ? 3 : 1);
   P.src_tab = p->src_tab && P.oblique && P.src_on ? (const T *)p->src_tab + (size_t)(p->src_off[s] + st) * row : nullptr;
-  P.src_fill = nullptr;
+  P.src_fill = 0;
   if (p->src_rows && P.oblique && P.src_on) {
     const int j = (st - first) % SRC_ROWS;
     P.src_tab = (const T *)(p->src_rows + j * row);
-    if (j == 0) P.src_fill = p->src_rows;
-    P.st = st;
-    P.tau = p->tau;
+    P.src_fill = j == 0;
   }
 }
 
@@ -402,6 +403,7 @@ StepLaunch<T, 1> single_launch(const StepParams<T> &P, const CUtensorMap &cur, c
   L.items = P.kz == p->items_kz ? p->items : nullptr;
   L.n_items = p->n_items;
   L.tile_w = p->tile.w;
+  L.tau = p->tau;
   L.chained = chained;
   L.p[0] = P;
   return L;
@@ -508,6 +510,7 @@ void launch_groups(ddfd_batch *b, bool adj, const std::vector<int> &idx, const C
     L.items = tab ? tables->d[gi] : nullptr;
     L.n_items = tab ? tables->n_items[gi] : 0;
     L.tile_w = b->tile.w;
+    L.tau = b->m[0]->tau;
     L.chained = chained || g0 > 0;
     for (int g = 0; g < L.nprob; ++g) {
       ddfd_problem *p = b->m[idx[g0 + g]];

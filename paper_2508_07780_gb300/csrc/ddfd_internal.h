@@ -100,12 +100,10 @@ struct StepParams {
   const T *hist_r;       // adjoint: hist[k]
   long long hcs;
   int hx, hp, hvec;
-  // oblique source of this step, tabulated (null: evaluated in the kernel): FP32 the three components' flux terms [3][n][px], FP64 the
-  // pulse times src_scale [n][px]
+  int src_fill;          // FP32: src_tab begins the flux of SRC_ROWS steps, to be evaluated before this one
+  // oblique source of this step, tabulated (null: evaluated in the kernel): FP32 the
+  // three components' flux terms [3][n][px], FP64 the pulse times src_scale [n][px]
   const T *src_tab;
-  float *src_fill;       // FP32: the table of SRC_ROWS steps that this step begins, to be filled before it (else null)
-  int st;                // ... its step and the time step
-  double tau;
   double *gacc_e;        // adjoint: gradient accumulators (FP64)
   double *gacc_s;
   // element-by-element FEM rows (fem_kind = DDFD_FEM_EBE): when ebe_r is set,
@@ -144,6 +142,7 @@ struct StepLaunch {
   int tile_w;  // FP64: width of the tile (Tile64)
   int chained; // the work before this launch in its stream is a kernel: launch as its dependent (launch_chained)
   StepParams<T> p[NB];
+  double tau;  // time step (last: ahead of p it costs the batch kernels registers)
 };
 
 // Tiles per axis of the FP32 step kernels' launch grid (32 x 16 tiles, with
