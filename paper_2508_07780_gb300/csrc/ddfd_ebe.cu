@@ -378,18 +378,18 @@ __global__ void __launch_bounds__(EBE_THREADS, EBE_CTAS) k_ebe(const __grid_cons
 static int g_ebe_ctas = 0;  // EBE_CTAS per SM
 
 template <typename T>
-void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s, bool chained) {
+void launch_ebe(const EbeParams<T> &P, int rb, bool adj, cudaStream_t s, bool chained) {
   const int want = std::max(P.n_blocks, (P.kuhn.n_list + 31) / 32);
   if (want <= 0) return;
   const int grid = std::min(want, g_ebe_ctas > 0 ? g_ebe_ctas : 1);
   const size_t smem = 128 + 2 * (size_t)P.stage_bytes;
-  const auto kernel = P.rb > EBE_RB ? (adj ? k_ebe<T, true, EBE_RB_TIGHT> : k_ebe<T, false, EBE_RB_TIGHT>)
+  const auto kernel = rb > EBE_RB ? (adj ? k_ebe<T, true, EBE_RB_TIGHT> : k_ebe<T, false, EBE_RB_TIGHT>)
                                     : (adj ? k_ebe<T, true, EBE_RB> : k_ebe<T, false, EBE_RB>);
   launch_chained(kernel, dim3((unsigned)grid), EBE_THREADS, smem, s, chained, P);
 }
 
-template void launch_ebe<float>(const EbeParams<float> &, bool, cudaStream_t, bool);
-template void launch_ebe<double>(const EbeParams<double> &, bool, cudaStream_t, bool);
+template void launch_ebe<float>(const EbeParams<float> &, int, bool, cudaStream_t, bool);
+template void launch_ebe<double>(const EbeParams<double> &, int, bool, cudaStream_t, bool);
 
 template <typename T, int RB>
 static cudaError_t set_ebe_smem(int lim) {

@@ -425,7 +425,6 @@ void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, 
   E.blk_nodes = p->ebe_blk_nodes;
   E.blk_rows = p->ebe_blk_rows;
   E.stage_bytes = p->ebe_smem;
-  E.rb = p->ebe_rb;
   E.err = err ? err : p->errflag;
   E.spin_limit = p->test_spin ? p->test_spin : 1u << 22;
   E.test_skip_copy = p->test_fault;
@@ -455,7 +454,7 @@ void enqueue_ebe(ddfd_problem *p, const void *field, bool adj, cudaStream_t sm, 
   E.xs = (const T *)p->xcoef;
   E.n_new = p->n_new;
   if (p->ebe_nblocks > 0 || p->kuhn_n > 0) {
-    launch_ebe<T>(E, adj, sm, chained);
+    launch_ebe<T>(E, p->ebe_rb, adj, sm, chained);
     ++*nk;
   }
 }

@@ -263,7 +263,6 @@ struct EbeParams {
   const unsigned char *blob;
   const int *blk_nodes;     // padded node offsets of the blocks' nodes
   const int *blk_rows;      // row indices of the blocks' rows
-  int rb;                   // rows that the blocks' incidence tables have room for
   int stage_bytes;          // shared memory of one pipeline stage (>= every block's)
   int *err;                 // bit 8: a bounded wait for a block's copy gave up
   uint32_t spin_limit;      // polls per bounded wait
@@ -294,9 +293,10 @@ void launch_copy_fem_nodes(const T *E, T *dst, int n, int px, long long cs, int 
 template <typename T>
 void launch_grad_literal(const T *Efem, const T *mu, double *gacc, int n, int px, long long cs, int a, int b,
                          double r2, cudaStream_t s);
+// rb: rows that the blocks' incidence tables have room for (EBE_RB or EBE_RB_TIGHT);
 // chained: the work before on `s` is a kernel (launch_chained)
 template <typename T>
-void launch_ebe(const EbeParams<T> &P, bool adj, cudaStream_t s, bool chained);
+void launch_ebe(const EbeParams<T> &P, int rb, bool adj, cudaStream_t s, bool chained);
 
 // Update of the new nodes of a refined FEM mesh (their rows are FEM rows
 // computed by k_ebe; interior nodes: no boundary or source terms), with the
