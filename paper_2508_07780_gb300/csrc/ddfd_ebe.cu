@@ -132,15 +132,21 @@ __device__ __forceinline__ void ebe_issue_nodes(const EbeParams<T> &P, const Ebe
 // The gather's thread blocks do them while their first copies are in flight
 // (as a launch of their own they took 4 us of a 21 us step of the 81^3 mesh).
 template <typename T, bool ADJ>
-__device__ __forceinline__ void kuhn_rows(const KuhnRowParams<T> &P) {
+__device__ __forceinline__ void kuhn_rows(const KuhnRowParams<T> &P, bool even) {
   const long long sx = 1, sy = P.px, sz = (long long)P.px * P.n;
   const long long off[7] = {sx, sy, sz, sx + sy, sx + sz, sy + sz, sx + sy + sz};
-  // a warp takes 32 rows in a row, neighbouring warps' rows go to neighbouring thread
-  // blocks: in FP64 the rows are bound by the SMs' FP64 units and have to spread over all
-  // of them (61^3 with a refined 31^3 cube, FP64: 106 / 90 -> 71 / 72 us a step; FP32 81^3,
-  // 41^3 cube: 19.4 / 21.0 -> 18.2 / 19.7)
-  const int warp = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
-  for (int q = 32 * warp + (int)(threadIdx.x & 31); q < P.n_list; q += (int)gridDim.x * EBE_THREADS) {
+  // Consecutive rows, which share operands in L1: an even share for every thread block.  In
+  // FP64 the rows are bound by the SMs' FP64 units and have to spread over all of them (61^3
+  // with a refined 31^3 cube, FP64: 106 / 90 us a step with 512 rows a block on the first 46,
+  // now 67 / 66; FP32 81^3, refined 41^3 cube, 17.3 / 18.4, now 15.7 / 17.4).  FP32 launches
+  // of several rounds of blocks keep 512 a block (121^3, refined 61^3 cube: 75.6 / 95.4, with
+  // even shares 75.8 / 96.2).
+  const int share = even ? ((P.n_list + (int)gridDim.x - 1) / (int)gridDim.x + 31) & ~31 : EBE_THREADS;
+  const int skip = share * ((int)gridDim.x - 1);  // to the block's next share
+  int end = share * ((int)blockIdx.x + 1);
+  for (int q = share * (int)blockIdx.x + (int)threadIdx.x;; q += EBE_THREADS) {
+    while (q >= end) q += skip, end += share * (int)gridDim.x;
+    if (q >= P.n_list) break;
     const int r = P.list[q];
     const long long o = P.row_node[r];
     T lap[3], g[3] = {T(0), T(0), T(0)};
@@ -201,7 +207,7 @@ __global__ void __launch_bounds__(EBE_THREADS, EBE_CTAS) k_ebe(const __grid_cons
   pdl_launch_dependents();
   pdl_wait();
   if (bi < P.n_blocks) ebe_issue_nodes<T, ADJ>(P, B, stage(0));
-  kuhn_rows<T, ADJ>(P.kuhn);
+  if (P.kuhn.n_list > 0) kuhn_rows<T, ADJ>(P.kuhn, sizeof(T) == 8 || P.n_blocks <= (int)gridDim.x);
   for (; bi < P.n_blocks; bi += gridDim.x) {
     cp_async_wait_all();
     if (tid == 0) s_ok = mbar_wait_bounded(bar + st, (parity >> st) & 1u, P.spin_limit) ? 1 : 0;
