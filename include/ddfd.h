@@ -107,7 +107,9 @@ typedef struct {
                             results are bitwise those of the full history) */
   int32_t cfl_check;     /* nonzero: estimate the stability bound by power iteration
                             at ddfd_set_coeffs and fail with DDFD_E_CFL above it */
-  int64_t mem_budget;    /* device bytes the handle may allocate; 0 = no limit */
+  int64_t mem_budget;    /* device bytes the handle may allocate; 0 = no limit.  Layouts
+                            that take more memory for speed are used where they fit at
+                            creation */
   int32_t tile_kz;       /* z planes per thread block of the step kernel's full items (FP32
                             tiles holding FEM-cube or free nodes; every FP64 tile); tuning:
                             0 = library default (FP32 2..24, FP64 1..12 planes: few enough

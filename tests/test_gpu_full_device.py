@@ -3,7 +3,8 @@ where they fit, and a handle that fits only without the padding still has to be
 created.  The device is filled with one buffer up to halfway between the bytes that
 the handle needs unpadded (those of the same handle with a memory budget, which never
 pads) and padded."""
-import numpy as np
+import gc
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -32,6 +33,7 @@ def test_a_handle_that_fits_only_unpadded_is_created(batched):
     h = make(mem_budget=1 << 40)
     need = h.get_info().device_bytes
     h.close()
+    gc.collect()  # (what earlier tests left would be freed between the two calls)
     torch.cuda.empty_cache()
     fill = torch.cuda.mem_get_info()[0] - need - more // 2
     assert fill > 0
