@@ -403,7 +403,6 @@ StepLaunch<T, 1> single_launch(const StepParams<T> &P, const CUtensorMap &cur, c
   L.items = P.kz == p->items_kz ? p->items : nullptr;
   L.n_items = p->n_items;
   L.tile_w = p->tile.w;
-  L.tau = p->tau;
   L.chained = chained;
   L.p[0] = P;
   return L;
@@ -509,7 +508,6 @@ void launch_groups(ddfd_batch *b, bool adj, const std::vector<int> &idx, const C
     L.items = tab ? tables->d[gi] : nullptr;
     L.n_items = tab ? tables->n_items[gi] : 0;
     L.tile_w = b->tile.w;
-    L.tau = b->m[0]->tau;
     L.chained = chained || g0 > 0;
     for (int g = 0; g < L.nprob; ++g) {
       ddfd_problem *p = b->m[idx[g0 + g]];

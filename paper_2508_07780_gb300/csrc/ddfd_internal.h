@@ -142,7 +142,6 @@ struct StepLaunch {
   int tile_w;  // FP64: width of the tile (Tile64)
   int chained; // the work before this launch in its stream is a kernel: launch as its dependent (launch_chained)
   StepParams<T> p[NB];
-  double tau;  // time step (last: ahead of p it costs the batch kernels registers)
 };
 
 // Tiles per axis of the FP32 step kernels' launch grid (32 x 16 tiles, with

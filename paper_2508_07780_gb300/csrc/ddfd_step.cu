@@ -856,13 +856,13 @@ static int launch_step(const StepLaunch<double, NB> &L, cudaStream_t s) {
 // 13.7 / 19.9 / 34.9 -> 6.5 / 12.0 / 25.2; one step at a time 6.2 / 17.5 / 26.1; a table
 // of every step 5.0 / 8.2 / 19.9).
 template <int NB>
-__global__ void __launch_bounds__(128) k_source_rows(const __grid_constant__ StepLaunch<float, NB> L, int st) {
+__global__ void __launch_bounds__(128) k_source_rows(const __grid_constant__ StepLaunch<float, NB> L, int st, double tau) {
   pdl_launch_dependents();
   const StepParams<float> &P = L.p[NB == 1 ? 0 : blockIdx.y];
   const int n = P.n, q = (int)(blockIdx.x * 128 + threadIdx.x), j = q / (n * n), d = q - j * n * n, y = d / n, x = d - n * y;
   const bool mine = j < SRC_ROWS && P.src_fill;
   double v = 0.0;
-  if (mine) v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width, __dmul_rn((double)(st + j), L.tau) - P.delay[d]);
+  if (mine) v = P.src_scale * pulse_value(P.pulse_kind, P.freq, P.t0, P.width, __dmul_rn((double)(st + j), tau) - P.delay[d]);
   pdl_wait();  // (the step before reads the table)
   if (mine)
     for (int c = 0; c < 3; ++c) const_cast<float *>(P.src_tab)[x + P.px * (y + (long long)n * (3 * j + c))] = (float)(P.pol[c] * v);
@@ -874,8 +874,9 @@ static int launch_step(const StepLaunch<float, NB> &L, cudaStream_t s) {
   for (int q = 0; q < L.nprob && !ADJ; ++q) rows |= L.p[q].src_fill != 0;
   if (rows) {
     const int total = L.p[0].n * L.p[0].n * SRC_ROWS;
+    const double tau = std::sqrt(L.p[0].tau2);  // (exactly: the root of a rounded square)
     launch_chained(k_source_rows<NB>, dim3((unsigned)((total + 127) / 128), (unsigned)L.nprob), 128, 0, s, L.chained != 0, L,
-                   (int)std::lround(L.p[0].t_n / L.tau));
+                   (int)std::lround(L.p[0].t_n / tau), tau);
     StepLaunch<float, NB> M = L;
     for (int q = 0; q < L.nprob; ++q) M.p[q].src_fill = 0;
     M.chained = 1;
